@@ -98,7 +98,9 @@ struct WalkParams {
     unsigned long long max_events;
     int reflect;
     int claim_static;                 // 1: static per-thread photon split
-    unsigned claim_chunk;             // photon ids a warp claims per global atomic (>= 32)
+    unsigned claim_chunk;             // photon ids a warp claims per global atomic (>= lanes)
+    unsigned lanes, warps;            // lanes per warp and warps per block that take photons;
+                                      // set at the launch
     const BatchSim *sims;             // batch: [n_sims], ordered by `first`
     int n_sims;
 };

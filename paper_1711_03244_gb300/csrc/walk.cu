@@ -25,11 +25,27 @@
 //  * The current medium's constants (scattering, absorption, time per length, g) sit in
 //    registers and are reloaded only when the photon enters another label; a photon's
 //    absorbed weight is formed once, from its final weight and roulette gains.
+//  * The walk is bound by instruction issue, and a warp issues the scattering code for 87%
+//    of its lanes but the face code for 13% (two spheres).  Lanes that reach a face
+//    therefore wait there while the others go on, so that the face code runs for several
+//    lanes at once.  Gate changes, the time limit, the event cap, the roulette and near-axial
+//    directions share one test per segment and a rarely taken path of their own, and one
+//    vote per round covers photons that ended and lanes without one: a scattering iteration
+//    takes about 140 warp instructions instead of 195.  Measured, against testing each
+//    condition in its own branch and crossing every face at once: two spheres, 2e7 photons
+//    175.6 -> 147 ms; layered tissue, 1e7 photons 87.0 -> 83.2 ms; 24 uneven batched
+//    simulations 57.6 -> 48.8 ms; cube, 3e5 photons 12.8 -> 9.5 ms.
+//  * A run with fewer photons than the grid has lanes gives each block its share: as few
+//    warps as hold it.  Its time is that of the longest history, whose warp then neither
+//    waits for warps beside it nor sits on an SM that took most of the photons
+//    (cube, 2e3 / 2e4 / 5e4 / 1e5 photons: 3.5 / 4.5 / 6.3 / 8.2 -> 2.9 / 4.0 / 4.8 / 7.5 ms;
+//    spreading them over all warps, a few lanes each, was slower: 5.2 ms at 2e4).
 //  * Fast hardware math (MUFU ex2/lg2/sin/cos/rsqrt/rcp) in the FP32 path, the CUDA
 //    analogue of the paper's "native" math optimisation; the same kernel instantiated in
 //    FP64 serves as the trajectory-parity diagnostic.
 #include <cfloat>
 #include <cstdint>
+#include <type_traits>
 
 #include "mcx_internal.h"
 
@@ -37,7 +53,14 @@ namespace mcxg {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-enum { EV_FACE = 0, EV_SCAT = 1, EV_TIME = 2 };
+// What a lane does next: take a segment, cross the voxel face it has reached, nothing (no
+// photon is left), take a new photon; kOver + fate: its photon has ended.
+enum { kWalk = 0, kFace = 1, kDone = 2, kIdle = 3, kOver = 8 };
+// A warp goes on with segments, its lanes at faces waiting, while at least kStay / 32 of its
+// lanes with a photon can take one.  Measured (1e7 photons, ms): two spheres, 13% of the
+// segments end at a face, 73.9 / 73.2 / 73.4 at 22 / 24 / 26 and 95 at 33 (no waiting);
+// layered tissue, 30% of them, 82.8 / 83.3 / 84.7.
+constexpr int kStay = 24;
 
 // ------------------------------------------------------------------------------ math
 template <typename R> struct M;
@@ -46,6 +69,9 @@ template <typename R> struct M;
 // is one lg2 and an attenuation one ex2 on the special-function unit; the FP64 walk uses
 // natural units and the library log/exp.
 template <> struct M<float> {
+    // one rounding each, never contracted into a neighbour
+    static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+    static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
     static __device__ __forceinline__ float log(float x) { return __logf(x); }
     static __device__ __forceinline__ float hop(float u)
     {
@@ -70,6 +96,8 @@ template <> struct M<float> {
     static __device__ __forceinline__ float tiny_hop() { return 1e-12f; }
 };
 template <> struct M<double> {
+    static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+    static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
     static __device__ __forceinline__ double log(double x) { return ::log(x); }
     static __device__ __forceinline__ double hop(double u) { return -::log(u); }
     static __device__ __forceinline__ double attenuation(double a, double l) { return ::exp(-a * l); }
@@ -170,16 +198,15 @@ template <typename R>
 __device__ __forceinline__ void hg_sample(const MedB<R> &B, R xi, R &ct, R &st)
 {
     const R inv_d = R(1) / (B.one_m_g + B.two_g * xi);
-    const R f = B.one_m_g2 * inv_d;
-    const R omc = B.one_m_g * (R(1) - xi) * (f + B.one_m_g) * inv_d;
-    const R opc = B.one_p_g * xi * (B.one_p_g + f) * inv_d;
-    ct = R(0.5) * (opc - omc);
+    // f = one_m_g2 inv_d stays inside the fused sums; (1 - xi) (1 - g) as one fused product
+    const R m1 = M<R>::mul(fma(-xi, B.one_m_g, B.one_m_g), fma(B.one_m_g2, inv_d, B.one_m_g));
+    const R m2 = M<R>::mul(M<R>::mul(B.one_p_g, xi), fma(B.one_m_g2, inv_d, B.one_p_g));
+    const R omc = M<R>::mul(m1, inv_d), opc = M<R>::mul(m2, inv_d);
+    ct = R(0.5) * M<R>::add(opc, -omc);
     st = M<R>::sqrt(omc * opc);
 }
 
-// The Henyey-Greenstein constants of anisotropy g; the host's table rounds them alike
-// (1 - g^2 as one fused multiply-add), so a walk that derives them from a g kept in a
-// register follows the same trajectories as one that reads the table.
+// The Henyey-Greenstein constants of anisotropy g (1 - g^2 as one fused multiply-add).
 template <typename R>
 __host__ __device__ __forceinline__ MedB<R> hg_consts(R g)
 {
@@ -187,21 +214,26 @@ __host__ __device__ __forceinline__ MedB<R> hg_consts(R g)
 }
 
 // MCML rotation of unit vector u by deflection (cos ct, sin st) and azimuth (sp, cp).
-template <typename R>
+// POLE = false leaves out the axis-aligned case (the caller has excluded it).  Products and
+// sums are written so that one rounding is possible for each: every instantiation then
+// rounds alike and follows the same trajectories.
+template <typename R, bool POLE = true>
 __device__ __forceinline__ void rotate(R &ux, R &uy, R &uz, R ct, R st, R sp, R cp)
 {
-    if (fabs(uz) > R(1) - R(1e-5)) {
+    if (POLE && fabs(uz) > R(1) - R(1e-5)) {
         ux = st * cp;
         uy = st * sp;
         uz = uz > R(0) ? ct : -ct;
     } else {
         // 1 - uz^2 evaluated as ux^2 + uy^2: no cancellation near the poles in FP32
-        const R one_m_uz2 = ux * ux + uy * uy;
+        const R one_m_uz2 = fma(uy, uy, M<R>::mul(ux, ux));
         const R rt = M<R>::rsqrt(one_m_uz2);          // 1 / sqrt(1 - uz^2)
-        const R a = st * rt;
-        const R nx = a * (ux * uz * cp - uy * sp) + ux * ct;
-        const R ny = a * (uy * uz * cp + ux * sp) + uy * ct;
-        const R nz = -st * cp * (one_m_uz2 * rt) + uz * ct;
+        const R a = M<R>::mul(st, rt);
+        const R px = fma(M<R>::mul(ux, uz), cp, -M<R>::mul(uy, sp));
+        const R py = fma(ux, sp, M<R>::mul(M<R>::mul(uy, uz), cp));
+        const R nx = fma(ux, ct, M<R>::mul(a, px));
+        const R ny = fma(uy, ct, M<R>::mul(a, py));
+        const R nz = fma(uz, ct, M<R>::mul(M<R>::mul(-st, cp), M<R>::mul(one_m_uz2, rt)));
         ux = nx;
         uy = ny;
         uz = nz;
@@ -359,7 +391,12 @@ walk_kernel(const WalkParams p)
     };
     const unsigned max_ev = p.max_events < 0xffffffffull ? (unsigned)p.max_events : 0xffffffffu;
 
-    bool alive = false, done = false;
+    int state = kIdle;
+    // a short run's photons go to the first p.lanes lanes of p.warps warps per block, which
+    // rotate with the block so that an SM's blocks use all of its schedulers
+    const unsigned wpb = blockDim.x >> 5;
+    const bool active = ((threadIdx.x >> 5) + blockIdx.x + (blockIdx.x >> 2)) % wpb < p.warps;
+    if (lane >= p.lanes) state = kDone;
     unsigned long long pid = ~0ull;   // current (or last) photon id; none yet
     Rng rng;
     rng.x = rng.y = 0;
@@ -371,19 +408,25 @@ walk_kernel(const WalkParams p)
     R w = 0, t = 0, s = 0, gained = 0, Lcur = 0, acc = 0;
     unsigned gate = 0;            // time gate of the current deposit run
     R t_next = 0;                 // time at which the gate advances
-    // the current medium's segment constants, reloaded only when the label changes (kept in
-    // registers: measured 5% faster at C2 than a shared-memory lookup in every segment); the
-    // compensated mode, whose block tile needs those registers, looks them up per segment
-    constexpr bool KEEP_MED = ACC != kAccCompensated;
+    const R t_safe = C.t_end * R(1.0 - 1e-5);
+    // a segment that ends before t_chk can neither start in a new gate nor meet the time
+    // limit: t_safe lies 1e-5 below the limit, far more than the roundings of a segment's time
+    R t_chk = 0;
+    // the current medium's constants, reloaded only when the label changes.  Kept in registers:
+    // against a shared-memory lookup in every segment, 5% less time for the two spheres, and
+    // with the scattering constants another 3%; in the compensated mode, whose block tile
+    // takes more registers, 11.9 -> 10.1 ms (cube, 3e5 photons) and 21.8 -> 21.4 ms (B1, 1e7)
     MedA<R> A_cur{};
     R tpl_cur = 0;                // its time per unit length
-    R g_cur = 0;                  // its anisotropy (the scattering constants follow from it)
-    unsigned nscat = 0, nrr = 0, c_face = 0, c_fres = 0, c_flush = 0, c_rr = 0;
+    MedB<R> B_cur{};              // its Henyey-Greenstein constants
+    unsigned nev = 0, nrr = 0, c_face = 0, c_fres = 0, c_flush = 0, c_rr = 0;
     float Lpath[DET ? kMaxDetMedia : 1];
 
     unsigned long long pool_next = 0;
     unsigned pool_left = 0;
     const unsigned last_gate = p.n_gates - 1u;
+    int axis = 0;                 // the axis of the face that ends the lane's segment
+    int again = 1;                // walking lanes with which the warp goes on with segments
 
     // a6/a12: one accumulation per (gate, voxel) run of deposits
     auto flush = [&]() {
@@ -430,373 +473,409 @@ walk_kernel(const WalkParams p)
         s = h > M<R>::tiny_hop() ? h : M<R>::tiny_hop();
     };
 
-    while (true) {
-        if (__any_sync(kFull, !alive)) {
-            // ---- a1: claim photon ids for lanes without a photon (one atomic per 32 ids)
-            const unsigned need = __ballot_sync(kFull, !alive && !done);
-            if (need) {
-                const unsigned n = __popc(need);
-                const unsigned rank = __popc(need & lt_mask);
-                unsigned long long id;
-                if (STATIC) {
-                    // the paper's thread-level split: thread g of T takes g, g + T, g + 2T,
-                    // ...; the next id follows from the lane's previous one
-                    const unsigned long long g0 = blockIdx.x * blockDim.x + threadIdx.x;
-                    id = pid == ~0ull ? g0 : pid - p.photon_offset + gridDim.x * blockDim.x;
-                } else if (pool_left >= n) {
-                    id = pool_next + rank;
-                    pool_next += n;
-                    pool_left -= n;
+    // a10/a11/a4: Henyey-Greenstein scattering, Russian roulette, the next hop.  CAREFUL:
+    // with the near-axial rotation and the roulette, which the other form leaves out
+    auto scatter = [&](auto careful) {
+        constexpr bool CAREFUL = decltype(careful)::value;
+        const MedB<R> &B = B_cur;
+        float u_hop, xi_hg, xi_phi;
+        rng.triple(u_hop, xi_hg, xi_phi);
+        R ct, st;
+        hg_sample(B, R(xi_hg), ct, st);
+        R sn, cs;
+        M<R>::sincos_2pi(R(xi_phi), &sn, &cs);
+        rotate<R, CAREFUL>(ux, uy, uz, ct, st, sn, cs);
+        iux = inv_dir(ux); iuy = inv_dir(uy); iuz = inv_dir(uz);
+        if constexpr (CAREFUL) {
+            if (w < C.rr_threshold) {
+                ++c_rr;
+                if (R(rng.uniform()) < C.rr_inv_m) {
+                    if constexpr (BATCH)
+                        atomicAdd(p.sims[sim].tally + MCX_TALLY_RR_GAINED, double((C.rr_m - R(1)) * w));
+                    else
+                        atomicAdd(&s_tally[MCX_TALLY_RR_GAINED], double((C.rr_m - R(1)) * w));
+                    gained += (C.rr_m - R(1)) * w;
+                    w *= C.rr_m;
+                    ++nrr;
                 } else {
-                    unsigned long long nb = 0;
-                    if (lane == 0) nb = atomicAdd(p.photon_counter, (unsigned long long)p.claim_chunk);
-                    nb = __shfl_sync(kFull, nb, 0);
-                    id = rank < pool_left ? pool_next + rank : nb + (rank - pool_left);
-                    const unsigned used_new = n - pool_left;
-                    pool_next = nb + used_new;
-                    pool_left = p.claim_chunk - used_new;
+                    state = kOver + MCX_FATE_ROULETTE;
                 }
-                if ((need >> lane) & 1u) {
-                    if (id >= p.n_photons) {
-                        done = true;
+            }
+        }
+        const R h = M<R>::hop(R(u_hop));
+        s = h > M<R>::tiny_hop() ? h : M<R>::tiny_hop();
+    };
+
+    if (active) while (true) {
+        if (__any_sync(kFull, state >= kIdle)) {
+            if (state >= kOver) {
+                // ---- photon finished: flush the deposit run, tallies, logs, detectors (a9, a12)
+                const int fate = state - kOver;
+                const unsigned nscat = nev - c_face;          // every counted segment ends in either
+                flush();
+                const R absorbed = R(1) + gained - w;
+                const int slot = fate == MCX_FATE_ESCAPED ? MCX_TALLY_ESCAPED
+                               : (fate == MCX_FATE_ROULETTE ? MCX_TALLY_RR_KILLED : MCX_TALLY_TIME);
+                if constexpr (BATCH) {
+                    atomicAdd(p.sims[sim].tally + slot, double(w));
+                    atomicAdd(p.sims[sim].tally + MCX_TALLY_ABSORBED, double(absorbed));
+                } else {
+                    atomicAdd(&s_tally[slot], double(w));
+                    atomicAdd(&s_tally[MCX_TALLY_ABSORBED], double(absorbed));
+                }
+                atomicAdd(&s_stats[MCX_STAT_SCATTER], (unsigned long long)nscat);
+                atomicAdd(&s_stats[MCX_STAT_FACE], (unsigned long long)c_face);
+                atomicAdd(&s_stats[MCX_STAT_FRESNEL], (unsigned long long)c_fres);
+                atomicAdd(&s_stats[MCX_STAT_FLUSH], (unsigned long long)c_flush);
+                atomicAdd(&s_stats[MCX_STAT_ROULETTE], (unsigned long long)c_rr);
+                atomicAdd(&s_stats[MCX_STAT_PHOTONS], 1ull);
+                if (fate == MCX_FATE_CAPPED) {
+                    atomicAdd(&s_stats[MCX_STAT_CAPPED], 1ull);
+                    atomicOr(p.status, kStatusCapped);
+                }
+                if constexpr (PAD && ACC != kAccCompensated) {
+                    // the voxel's indices from its linear index in the padded volume
+                    const unsigned r = vlin % G_sz;
+                    iz = (int)(vlin / G_sz) - 1;
+                    iy = (int)(r / G_sy) - 1;
+                    ix = (int)(r % G_sy) - 1;
+                }
+                const R hh = R(p.h);
+                const R ex = (R(ix) + qx) * hh, ey = (R(iy) + qy) * hh, ez = (R(iz) + qz) * hh;
+                const unsigned long long rel = pid - p.photon_offset;
+                if (rel < p.exit_log) {
+                    mcx_exit e;
+                    e.fate = fate; e.nscat = nscat;
+                    e.pos[0] = float(ex); e.pos[1] = float(ey); e.pos[2] = float(ez);
+                    e.dir[0] = float(ux); e.dir[1] = float(uy); e.dir[2] = float(uz);
+                    e.w = float(w); e.t = float(t);
+                    p.exits[rel] = e;
+                }
+                if (DET && fate == MCX_FATE_ESCAPED) {
+                    const float vx = float(R(ix) + qx), vy = float(R(iy) + qy), vz = float(R(iz) + qz);
+                    for (int d = 0; d < p.n_det; ++d) {
+                        const float4 D = s_det[d];
+                        const float dx = vx - D.x, dy = vy - D.y, dz = vz - D.z;
+                        if (dx * dx + dy * dy + dz * dz <= D.w) {
+                            atomicAdd(&s_stats[MCX_STAT_DETECTED], 1ull);
+                            const unsigned long long slot_i = atomicAdd(p.det_count, 1ull);
+                            if (slot_i < p.max_detected) {
+                                if (lab < kMaxDetMedia) Lpath[lab] += float(Lcur);
+                                float *rec = p.det_buf + slot_i * (unsigned long long)p.rec_stride;
+                                rec[0] = __uint_as_float((unsigned)(pid & 0xffffffffull));
+                                rec[1] = __uint_as_float((unsigned)(pid >> 32));
+                                rec[2] = __int_as_float(d);
+                                rec[3] = __uint_as_float(nscat);
+                                rec[4] = float(w);
+                                rec[5] = float(ex); rec[6] = float(ey); rec[7] = float(ez);
+                                rec[8] = float(ux); rec[9] = float(uy); rec[10] = float(uz);
+                                rec[11] = __uint_as_float(nrr);
+                                for (int m = 1; m < p.n_media && m < kMaxDetMedia; ++m)
+                                    rec[kRecBase + m - 1] = Lpath[m] * p.h;
+                            } else {
+                                atomicOr(p.status, kStatusDetOverflow);
+                            }
+                            break;
+                        }
+                    }
+                }
+                state = kIdle;
+            }
+            __syncwarp();
+            // ---- a1: claim photon ids for lanes without a photon (one atomic per 32 ids)
+            const unsigned need = __ballot_sync(kFull, state == kIdle);
+            const unsigned n = __popc(need);
+            const unsigned rank = __popc(need & lt_mask);
+            unsigned long long id;
+            if (STATIC) {
+                // the paper's thread-level split: thread g of T takes g, g + T, g + 2T,
+                // ...; the next id follows from the lane's previous one
+                const unsigned long long g0 = blockIdx.x * blockDim.x + threadIdx.x;
+                id = pid == ~0ull ? g0 : pid - p.photon_offset + gridDim.x * blockDim.x;
+            } else if (pool_left >= n) {
+                id = pool_next + rank;
+                pool_next += n;
+                pool_left -= n;
+            } else {
+                unsigned long long nb = 0;
+                if (lane == 0) nb = atomicAdd(p.photon_counter, (unsigned long long)p.claim_chunk);
+                nb = __shfl_sync(kFull, nb, 0);
+                id = rank < pool_left ? pool_next + rank : nb + (rank - pool_left);
+                const unsigned used_new = n - pool_left;
+                pool_next = nb + used_new;
+                pool_left = p.claim_chunk - used_new;
+            }
+            if ((need >> lane) & 1u) {
+                if (id >= p.n_photons) {
+                    state = kDone;
+                } else {
+                    // ---- a2/a3: per-photon RNG and launch
+                    R px, py, pz, e1[3], e2[3], waist;
+                    int kind;
+                    if constexpr (BATCH) {
+                        // the simulation holding flattened index id: the last with first <= id
+                        int lo = 0, hi = p.n_sims - 1;
+                        while (lo < hi) {
+                            const int mid = (lo + hi + 1) >> 1;
+                            if (p.sims[mid].first <= id) lo = mid; else hi = mid - 1;
+                        }
+                        sim = lo;
+                        const BatchSim &S = p.sims[sim];
+                        pid = id - S.first;
+                        rng.seed(S.seed, pid);
+                        G_labels = S.labels; G_flu = S.fluence; G_flu64 = S.fluence64;
+                        G_nx = S.nx; G_ny = S.ny; G_nz = S.nz; G_nvox = S.nvox;
+                        G_sy = S.sy; G_sz = S.sz;
+                        tab0 = S.tab0;
+                        px = S.src_pos[0]; py = S.src_pos[1]; pz = S.src_pos[2];
+                        ux = S.src_dir[0]; uy = S.src_dir[1]; uz = S.src_dir[2];
+                        for (int a = 0; a < 3; ++a) { e1[a] = S.src_e1[a]; e2[a] = S.src_e2[a]; }
+                        waist = S.waist;
+                        kind = S.src_kind;
                     } else {
-                        // ---- a2/a3: per-photon RNG and launch
-                        R px, py, pz, e1[3], e2[3], waist;
-                        int kind;
-                        if constexpr (BATCH) {
-                            // the simulation holding flattened index id: the last with first <= id
-                            int lo = 0, hi = p.n_sims - 1;
-                            while (lo < hi) {
-                                const int mid = (lo + hi + 1) >> 1;
-                                if (p.sims[mid].first <= id) lo = mid; else hi = mid - 1;
-                            }
-                            sim = lo;
-                            const BatchSim &S = p.sims[sim];
-                            pid = id - S.first;
-                            rng.seed(S.seed, pid);
-                            G_labels = S.labels; G_flu = S.fluence; G_flu64 = S.fluence64;
-                            G_nx = S.nx; G_ny = S.ny; G_nz = S.nz; G_nvox = S.nvox;
-                            G_sy = S.sy; G_sz = S.sz;
-                            tab0 = S.tab0;
-                            px = S.src_pos[0]; py = S.src_pos[1]; pz = S.src_pos[2];
-                            ux = S.src_dir[0]; uy = S.src_dir[1]; uz = S.src_dir[2];
-                            for (int a = 0; a < 3; ++a) { e1[a] = S.src_e1[a]; e2[a] = S.src_e2[a]; }
-                            waist = S.waist;
-                            kind = S.src_kind;
-                        } else {
-                            pid = p.photon_offset + id;
-                            rng.seed(p.seed, pid);
-                            px = C.src_pos[0]; py = C.src_pos[1]; pz = C.src_pos[2];
-                            ux = C.src_dir[0]; uy = C.src_dir[1]; uz = C.src_dir[2];
-                            for (int a = 0; a < 3; ++a) { e1[a] = C.src_e1[a]; e2[a] = C.src_e2[a]; }
-                            waist = C.waist;
-                            kind = p.src_kind;
-                        }
-                        if (kind == 1) {
-                            float f1, f2;
-                            rng.pair(f1, f2);
-                            const R r = waist * M<R>::sqrt(-M<R>::log(R(f1)) * R(0.5));
-                            R sn, cs;
-                            M<R>::sincos_2pi(R(f2), &sn, &cs);
-                            px += r * (cs * e1[0] + sn * e2[0]);
-                            py += r * (cs * e1[1] + sn * e2[1]);
-                            pz += r * (cs * e1[2] + sn * e2[2]);
-                        }
-                        const R fx = floor(px), fy = floor(py), fz = floor(pz);
-                        ix = (int)fx - ((px == fx && ux < R(0)) ? 1 : 0);
-                        iy = (int)fy - ((py == fy && uy < R(0)) ? 1 : 0);
-                        iz = (int)fz - ((pz == fz && uz < R(0)) ? 1 : 0);
-                        qx = px - R(ix); qy = py - R(iy); qz = pz - R(iz);
-                        iux = inv_dir(ux); iuy = inv_dir(uy); iuz = inv_dir(uz);
-                        w = R(1); t = R(0); gained = R(0); Lcur = R(0); acc = R(0);
-                        gate = 0;
-                        t_next = last_gate > 0 ? C.dt : M<R>::huge();
-                        nscat = nrr = c_face = c_fres = c_flush = c_rr = 0;
-                        if (DET)
-                            for (int m = 0; m < p.n_media && m < kMaxDetMedia; ++m) Lpath[m] = 0.f;
-                        const bool inside = (unsigned)ix < (unsigned)G_nx &&
-                                            (unsigned)iy < (unsigned)G_ny &&
-                                            (unsigned)iz < (unsigned)G_nz;
-                        vlin = inside ? ((unsigned)iz * G_sz + (unsigned)iy * G_sy + (unsigned)ix +
-                                         (PAD ? G_sz + G_sy + 1u : 0u)) : 0u;
-                        lab = inside ? (int)__ldg(G_labels + vlin) : 0;
-                        if constexpr (KEEP_MED) {
-                            A_cur = medA(lab);
-                            tpl_cur = med_tpl(lab);
-                            g_cur = R(0.5) * medB(lab).two_g;      // 2g / 2: exact
-                        }
-                        alive = lab != 0;
-                        if (alive) {
-                            new_hop();
-                        } else {
-                            // launched outside the medium: counted as escaped, never enters
-                            if constexpr (BATCH) atomicAdd(p.sims[sim].tally + MCX_TALLY_ESCAPED, 1.0);
-                            else atomicAdd(&s_tally[MCX_TALLY_ESCAPED], 1.0);
-                            atomicAdd(&s_stats[MCX_STAT_PHOTONS], 1ull);
-                            const unsigned long long rel = pid - p.photon_offset;
-                            if (rel < p.exit_log) {
-                                mcx_exit e;
-                                e.fate = MCX_FATE_MISSED; e.nscat = 0;
-                                e.pos[0] = float(px * R(p.h)); e.pos[1] = float(py * R(p.h));
-                                e.pos[2] = float(pz * R(p.h));
-                                e.dir[0] = float(ux); e.dir[1] = float(uy); e.dir[2] = float(uz);
-                                e.w = 1.f; e.t = 0.f;
-                                p.exits[rel] = e;
-                            }
+                        pid = p.photon_offset + id;
+                        rng.seed(p.seed, pid);
+                        px = C.src_pos[0]; py = C.src_pos[1]; pz = C.src_pos[2];
+                        ux = C.src_dir[0]; uy = C.src_dir[1]; uz = C.src_dir[2];
+                        for (int a = 0; a < 3; ++a) { e1[a] = C.src_e1[a]; e2[a] = C.src_e2[a]; }
+                        waist = C.waist;
+                        kind = p.src_kind;
+                    }
+                    if (kind == 1) {
+                        float f1, f2;
+                        rng.pair(f1, f2);
+                        const R r = waist * M<R>::sqrt(-M<R>::log(R(f1)) * R(0.5));
+                        R sn, cs;
+                        M<R>::sincos_2pi(R(f2), &sn, &cs);
+                        px += r * (cs * e1[0] + sn * e2[0]);
+                        py += r * (cs * e1[1] + sn * e2[1]);
+                        pz += r * (cs * e1[2] + sn * e2[2]);
+                    }
+                    const R fx = floor(px), fy = floor(py), fz = floor(pz);
+                    ix = (int)fx - ((px == fx && ux < R(0)) ? 1 : 0);
+                    iy = (int)fy - ((py == fy && uy < R(0)) ? 1 : 0);
+                    iz = (int)fz - ((pz == fz && uz < R(0)) ? 1 : 0);
+                    qx = px - R(ix); qy = py - R(iy); qz = pz - R(iz);
+                    iux = inv_dir(ux); iuy = inv_dir(uy); iuz = inv_dir(uz);
+                    w = R(1); t = R(0); gained = R(0); Lcur = R(0); acc = R(0);
+                    gate = 0;
+                    t_next = last_gate > 0 ? C.dt : M<R>::huge();
+                    t_chk = t_next < t_safe ? t_next : t_safe;
+                    nev = nrr = c_face = c_fres = c_flush = c_rr = 0;
+                    if (DET)
+                        for (int m = 0; m < p.n_media && m < kMaxDetMedia; ++m) Lpath[m] = 0.f;
+                    const bool inside = (unsigned)ix < (unsigned)G_nx &&
+                                        (unsigned)iy < (unsigned)G_ny &&
+                                        (unsigned)iz < (unsigned)G_nz;
+                    vlin = inside ? ((unsigned)iz * G_sz + (unsigned)iy * G_sy + (unsigned)ix +
+                                     (PAD ? G_sz + G_sy + 1u : 0u)) : 0u;
+                    lab = inside ? (int)__ldg(G_labels + vlin) : 0;
+                    A_cur = medA(lab);
+                    tpl_cur = med_tpl(lab);
+                    B_cur = medB(lab);
+                    if (lab != 0) {
+                        state = kWalk;
+                        new_hop();
+                    } else {
+                        // launched outside the medium: counted as escaped, never enters
+                        if constexpr (BATCH) atomicAdd(p.sims[sim].tally + MCX_TALLY_ESCAPED, 1.0);
+                        else atomicAdd(&s_tally[MCX_TALLY_ESCAPED], 1.0);
+                        atomicAdd(&s_stats[MCX_STAT_PHOTONS], 1ull);
+                        const unsigned long long rel = pid - p.photon_offset;
+                        if (rel < p.exit_log) {
+                            mcx_exit e;
+                            e.fate = MCX_FATE_MISSED; e.nscat = 0;
+                            e.pos[0] = float(px * R(p.h)); e.pos[1] = float(py * R(p.h));
+                            e.pos[2] = float(pz * R(p.h));
+                            e.dir[0] = float(ux); e.dir[1] = float(uy); e.dir[2] = float(uz);
+                            e.w = 1.f; e.t = 0.f;
+                            p.exits[rel] = e;
                         }
                     }
                 }
             }
-            if (__all_sync(kFull, done)) break;
-            if (!alive) continue;
+            const unsigned live = __ballot_sync(kFull, state == kWalk);
+            if (!live && __all_sync(kFull, state == kDone)) break;
+            again = max(1, (__popc(live) * kStay + 31) >> 5);
         }
 
-        int fate = MCX_FATE_NONE;
-        if (nscat + c_face >= max_ev) {
-            fate = MCX_FATE_CAPPED;
-        } else {
-            // ---- a7: the gate of this segment's start (time only increases)
-            if (t >= t_next) {
-                flush();
-                unsigned g2 = (unsigned)(t * C.inv_dt);
-                g2 = g2 > gate + 1u ? g2 : gate + 1u;
-                gate = g2 < last_gate ? g2 : last_gate;
-                t_next = gate < last_gate ? R(gate + 1u) * C.dt : M<R>::huge();
-            }
-            const MedA<R> A = KEEP_MED ? A_cur : medA(lab);
-            const R tpl = KEEP_MED ? tpl_cur : med_tpl(lab);
-            // ---- a5: nearest face (lowest axis on ties), scattering point, time limit
-            const R dxf = face_dist(qx, iux);
-            const R dyf = face_dist(qy, iuy);
-            const R dzf = face_dist(qz, iuz);
-            // fmin ignores the NaN distance of a zero direction component
-            const R lmin = fmin(fmin(dxf, dyf), dzf);
-            const int ax = lmin == dxf ? 0 : (lmin == dyf ? 1 : 2);     // lowest axis on ties
-            R l = lmin > R(0) ? lmin : R(0);  // rounding past a face: a zero-length step onto it
-            int ev = EV_FACE;
-            const R dscat = s * A.inv_mus;
-            if (dscat <= l) { l = dscat; ev = EV_SCAT; }
-            R dtime = (C.t_end - t) * A.len_per_t;
-            dtime = dtime > R(0) ? dtime : R(0);
-            if (dtime <= l) { l = dtime; ev = EV_TIME; }
-
-            // ---- a5/a6: move, age, absorb into the current (gate, voxel) run
-            qx += l * ux;
-            qy += l * uy;
-            qz += l * uz;
-            t += l * tpl;
-            s -= l * A.mus;                   // a scattering event draws the next hop
-            if (DET) Lcur += l;
-            const R wn = w * M<R>::attenuation(A.mua, l);
-            const R dw = w - wn;
-            w = wn;
-            acc += dw;
-
-            if (ev == EV_TIME) {
-                fate = MCX_FATE_TIME;
-            } else if (ev == EV_FACE) {
-                // ---- a8: voxel face
-                ++c_face;
-                const bool p0 = ax == 0, p1 = ax == 1;
-                const R inv_a = p0 ? iux : (p1 ? iuy : iuz);
-                const bool up = inv_a > R(0);              // u_ax >= 0 (inv_dir of 0 is +huge)
-                const unsigned stride = p0 ? 1u : (p1 ? G_sy : G_sz);
-                const unsigned nlin = up ? vlin + stride : vlin - stride;
-                // per-axis index of the next voxel: tracked unless the border makes it
-                // unnecessary (the compensated mode's block tile still needs it)
-                constexpr bool AXES = !PAD || ACC == kAccCompensated;
-                int ia = 0;
-                if constexpr (AXES) ia = (p0 ? ix : (p1 ? iy : iz)) + (up ? 1 : -1);
-                int b;
-                if constexpr (PAD) {
-                    b = (int)__ldg(G_labels + nlin);
+        // ---- segments, until enough lanes wait at a face
+        do {
+            if (state == kWalk) {
+                const MedA<R> &A = A_cur;
+                const R tpl = tpl_cur;
+                // ---- a5: nearest face (lowest axis on ties), scattering point
+                const R dxf = face_dist(qx, iux);
+                const R dyf = face_dist(qy, iuy);
+                const R dzf = face_dist(qz, iuz);
+                // fmin ignores the NaN distance of a zero direction component
+                const R lmin = fmin(fmin(dxf, dyf), dzf);
+                axis = lmin == dxf ? 0 : (lmin == dyf ? 1 : 2);   // lowest axis on ties
+                R l = lmin > R(0) ? lmin : R(0);  // rounding past a face: a zero-length step onto it
+                const R dscat = s * A.inv_mus;
+                const bool sct = dscat <= l;
+                l = sct ? dscat : l;
+                R tn = t + l * tpl;
+                R wn = w * M<R>::attenuation(A.mua, l);
+                const bool capped = nev >= max_ev;
+                // gate change, time limit, event cap, roulette, near-axial direction: each
+                // photon meets these a few times in some thousand segments
+                const bool rare = !(tn < t_chk) | capped | (wn < C.rr_threshold) |
+                                  (fabs(uz) > R(1) - R(1e-5));
+                ++nev;
+                if (__builtin_expect(rare, 0)) {
+                    bool timed = false;
+                    if (capped) {
+                        --nev;
+                        state = kOver + MCX_FATE_CAPPED;
+                    } else {
+                        if (t >= t_next) {                // a7: the gate of this segment's start
+                            flush();
+                            unsigned g2 = (unsigned)(t * C.inv_dt);
+                            g2 = g2 > gate + 1u ? g2 : gate + 1u;
+                            gate = g2 < last_gate ? g2 : last_gate;
+                            t_next = gate < last_gate ? R(gate + 1u) * C.dt : M<R>::huge();
+                            t_chk = t_next < t_safe ? t_next : t_safe;
+                        }
+                        R dtime = (C.t_end - t) * medA(lab).len_per_t;
+                        dtime = dtime > R(0) ? dtime : R(0);
+                        if (dtime <= l) {
+                            l = dtime;
+                            timed = true;
+                            tn = t + l * tpl;
+                            wn = w * M<R>::attenuation(A.mua, l);
+                            --nev;
+                        }
+                        qx += l * ux;
+                        qy += l * uy;
+                        qz += l * uz;
+                        t = tn;
+                        s -= l * A.mus;
+                        if (DET) Lcur += l;
+                        const R dw = w - wn;
+                        w = wn;
+                        acc += dw;
+                        if (timed) state = kOver + MCX_FATE_TIME;
+                        else if (sct) scatter(std::true_type{});
+                        else state = kFace;
+                    }
                 } else {
-                    const int dim = p0 ? G_nx : (p1 ? G_ny : G_nz);
-                    b = (unsigned)ia < (unsigned)dim ? (int)__ldg(G_labels + nlin) : 0;
+                    // ---- a5/a6: move, age, absorb into the current (gate, voxel) run
+                    qx += l * ux;
+                    qy += l * uy;
+                    qz += l * uz;
+                    t = tn;
+                    s -= l * A.mus;                   // a scattering event draws the next hop
+                    if (DET) Lcur += l;
+                    const R dw = w - wn;
+                    w = wn;
+                    acc += dw;
+                    if (sct) scatter(std::false_type{});
+                    else state = kFace;
                 }
-                if (b == lab) {
-                    // same medium: straight into the next voxel, entering on the near face
-                    flush();                              // the deposit run ends with the voxel
-                    const R qn = up ? R(0) : R(1);
-                    qx = p0 ? qn : qx;
-                    qy = p1 ? qn : qy;
-                    qz = (!p0 && !p1) ? qn : qz;
+            }
+        } while (__popc(__ballot_sync(kFull, state == kWalk)) >= again);
+
+        if (state == kFace) {
+            // ---- a8: voxel face
+            state = kWalk;
+            ++c_face;
+            const bool p0 = axis == 0, p1 = axis == 1;
+            const R inv_a = p0 ? iux : (p1 ? iuy : iuz);
+            const bool up = inv_a > R(0);              // u_ax >= 0 (inv_dir of 0 is +huge)
+            const unsigned stride = p0 ? 1u : (p1 ? G_sy : G_sz);
+            const unsigned nlin = up ? vlin + stride : vlin - stride;
+            // per-axis index of the next voxel: tracked unless the border makes it
+            // unnecessary (the compensated mode's block tile still needs it)
+            constexpr bool AXES = !PAD || ACC == kAccCompensated;
+            int ia = 0;
+            if constexpr (AXES) ia = (p0 ? ix : (p1 ? iy : iz)) + (up ? 1 : -1);
+            int b;
+            if constexpr (PAD) {
+                b = (int)__ldg(G_labels + nlin);
+            } else {
+                const int dim = p0 ? G_nx : (p1 ? G_ny : G_nz);
+                b = (unsigned)ia < (unsigned)dim ? (int)__ldg(G_labels + nlin) : 0;
+            }
+            if (b == lab) {
+                // same medium: straight into the next voxel, entering on the near face
+                flush();                              // the deposit run ends with the voxel
+                const R qn = up ? R(0) : R(1);
+                qx = p0 ? qn : qx;
+                qy = p1 ? qn : qy;
+                qz = (!p0 && !p1) ? qn : qz;
+                if constexpr (AXES) {
+                    ix = p0 ? ia : ix;
+                    iy = p1 ? ia : iy;
+                    iz = (!p0 && !p1) ? ia : iz;
+                }
+                vlin = nlin;
+                if (s <= R(0)) new_hop();            // hop used up by rounding at the face
+            } else {
+                // photon on the face
+                const R qb = up ? R(1) : R(0);
+                qx = p0 ? qb : qx;
+                qy = p1 ? qb : qy;
+                qz = !p0 && !p1 ? qb : qz;
+                const R ua = p0 ? ux : (p1 ? uy : uz);
+                bool enter = false, escape = false;
+                if (!p.reflect) {
+                    // the paper's B1: the exterior terminates, internal mismatches pass
+                    if (b == 0) escape = true; else enter = true;
+                } else {
+                    const R na = med_n(lab), nb = med_n(b);
+                    if (na == nb) {
+                        if (b == 0) escape = true; else enter = true;
+                    } else {
+                        ++c_fres;
+                        const R ci = fabs(ua);
+                        const R eta = M<R>::div(na, nb);
+                        const R st2 = eta * eta * fma(-ci, ci, R(1));   // one rounding
+                        bool refl = true;                 // total internal reflection
+                        if (st2 < R(1)) refl = R(rng.uniform()) < fresnel(na, nb, ci, st2);
+                        if (refl) {
+                            ux = p0 ? -ux : ux;
+                            uy = p1 ? -uy : uy;
+                            uz = !p0 && !p1 ? -uz : uz;
+                            iux = p0 ? -iux : iux;
+                            iuy = p1 ? -iuy : iuy;
+                            iuz = !p0 && !p1 ? -iuz : iuz;
+                        } else {
+                            // Snell: tangential components x eta, normal = +-cos(theta_t)
+                            const R ctt = M<R>::sqrt(R(1) - st2);
+                            const R un = up ? ctt : -ctt;
+                            ux = p0 ? un : ux * eta;
+                            uy = p1 ? un : uy * eta;
+                            uz = !p0 && !p1 ? un : uz * eta;
+                            iux = inv_dir(ux); iuy = inv_dir(uy); iuz = inv_dir(uz);
+                            if (b == 0) escape = true; else enter = true;
+                        }
+                    }
+                }
+                if (enter) {
+                    flush();
                     if constexpr (AXES) {
                         ix = p0 ? ia : ix;
                         iy = p1 ? ia : iy;
-                        iz = (!p0 && !p1) ? ia : iz;
+                        iz = !p0 && !p1 ? ia : iz;
                     }
+                    qx = p0 ? R(1) - qb : qx;
+                    qy = p1 ? R(1) - qb : qy;
+                    qz = !p0 && !p1 ? R(1) - qb : qz;
                     vlin = nlin;
-                    if (s <= R(0)) new_hop();            // hop used up by rounding at the face
-                } else {
-                    // photon on the face
-                    const R qb = up ? R(1) : R(0);
-                    qx = p0 ? qb : qx;
-                    qy = p1 ? qb : qy;
-                    qz = !p0 && !p1 ? qb : qz;
-                    const R ua = p0 ? ux : (p1 ? uy : uz);
-                    bool enter = false, escape = false;
-                    if (!p.reflect) {
-                        // the paper's B1: the exterior terminates, internal mismatches pass
-                        if (b == 0) escape = true; else enter = true;
-                    } else {
-                        const R na = med_n(lab), nb = med_n(b);
-                        if (na == nb) {
-                            if (b == 0) escape = true; else enter = true;
-                        } else {
-                            ++c_fres;
-                            const R ci = fabs(ua);
-                            const R eta = M<R>::div(na, nb);
-                            const R st2 = eta * eta * fma(-ci, ci, R(1));   // one rounding
-                            bool refl = true;                 // total internal reflection
-                            if (st2 < R(1)) refl = R(rng.uniform()) < fresnel(na, nb, ci, st2);
-                            if (refl) {
-                                ux = p0 ? -ux : ux;
-                                uy = p1 ? -uy : uy;
-                                uz = !p0 && !p1 ? -uz : uz;
-                                iux = p0 ? -iux : iux;
-                                iuy = p1 ? -iuy : iuy;
-                                iuz = !p0 && !p1 ? -iuz : iuz;
-                            } else {
-                                // Snell: tangential components x eta, normal = +-cos(theta_t)
-                                const R ctt = M<R>::sqrt(R(1) - st2);
-                                const R un = up ? ctt : -ctt;
-                                ux = p0 ? un : ux * eta;
-                                uy = p1 ? un : uy * eta;
-                                uz = !p0 && !p1 ? un : uz * eta;
-                                iux = inv_dir(ux); iuy = inv_dir(uy); iuz = inv_dir(uz);
-                                if (b == 0) escape = true; else enter = true;
-                            }
-                        }
-                    }
-                    if (enter) {
-                        flush();
-                        if constexpr (AXES) {
-                            ix = p0 ? ia : ix;
-                            iy = p1 ? ia : iy;
-                            iz = !p0 && !p1 ? ia : iz;
-                        }
-                        qx = p0 ? R(1) - qb : qx;
-                        qy = p1 ? R(1) - qb : qy;
-                        qz = !p0 && !p1 ? R(1) - qb : qz;
-                        vlin = nlin;
-                        if (DET) {
-                            if (lab < kMaxDetMedia) Lpath[lab] += float(Lcur);
-                            Lcur = R(0);
-                        }
-                        lab = b;
-                        if constexpr (KEEP_MED) {
-                            A_cur = medA(b);
-                            tpl_cur = med_tpl(b);
-                            g_cur = R(0.5) * medB(b).two_g;
-                        }
-                    }
-                    if (escape) fate = MCX_FATE_ESCAPED;
-                    else if (s <= R(0)) new_hop();        // hop used up by rounding at the face
-                }
-            } else {
-                // ---- a10: Henyey-Greenstein scattering; a11: Russian roulette
-                ++nscat;
-                const MedB<R> B = KEEP_MED ? hg_consts(g_cur) : medB(lab);
-                float u_hop, xi_hg, xi_phi;
-                rng.triple(u_hop, xi_hg, xi_phi);
-                R ct, st;
-                hg_sample(B, R(xi_hg), ct, st);
-                R sn, cs;
-                M<R>::sincos_2pi(R(xi_phi), &sn, &cs);
-                rotate(ux, uy, uz, ct, st, sn, cs);
-                iux = inv_dir(ux); iuy = inv_dir(uy); iuz = inv_dir(uz);
-                if (w < C.rr_threshold) {
-                    ++c_rr;
-                    if (R(rng.uniform()) < C.rr_inv_m) {
-                        if constexpr (BATCH)
-                            atomicAdd(p.sims[sim].tally + MCX_TALLY_RR_GAINED, double((C.rr_m - R(1)) * w));
-                        else
-                            atomicAdd(&s_tally[MCX_TALLY_RR_GAINED], double((C.rr_m - R(1)) * w));
-                        gained += (C.rr_m - R(1)) * w;
-                        w *= C.rr_m;
-                        ++nrr;
-                    } else {
-                        fate = MCX_FATE_ROULETTE;
-                    }
-                }
-                if (fate == MCX_FATE_NONE) {              // a4: the next hop, drawn with the
-                    const R h = M<R>::hop(R(u_hop));      // deflection
-                    s = h > M<R>::tiny_hop() ? h : M<R>::tiny_hop();
-                }
-            }
-        }
-        if (fate == MCX_FATE_NONE) continue;
-
-        // ---- photon finished: flush the deposit run, tallies, logs, detectors (a9, a12)
-        flush();
-        const R absorbed = R(1) + gained - w;
-        const int slot = fate == MCX_FATE_ESCAPED ? MCX_TALLY_ESCAPED
-                       : (fate == MCX_FATE_ROULETTE ? MCX_TALLY_RR_KILLED : MCX_TALLY_TIME);
-        if constexpr (BATCH) {
-            atomicAdd(p.sims[sim].tally + slot, double(w));
-            atomicAdd(p.sims[sim].tally + MCX_TALLY_ABSORBED, double(absorbed));
-        } else {
-            atomicAdd(&s_tally[slot], double(w));
-            atomicAdd(&s_tally[MCX_TALLY_ABSORBED], double(absorbed));
-        }
-        atomicAdd(&s_stats[MCX_STAT_SCATTER], (unsigned long long)nscat);
-        atomicAdd(&s_stats[MCX_STAT_FACE], (unsigned long long)c_face);
-        atomicAdd(&s_stats[MCX_STAT_FRESNEL], (unsigned long long)c_fres);
-        atomicAdd(&s_stats[MCX_STAT_FLUSH], (unsigned long long)c_flush);
-        atomicAdd(&s_stats[MCX_STAT_ROULETTE], (unsigned long long)c_rr);
-        atomicAdd(&s_stats[MCX_STAT_PHOTONS], 1ull);
-        if (fate == MCX_FATE_CAPPED) {
-            atomicAdd(&s_stats[MCX_STAT_CAPPED], 1ull);
-            atomicOr(p.status, kStatusCapped);
-        }
-        if constexpr (PAD && ACC != kAccCompensated) {
-            // the voxel's indices from its linear index in the padded volume
-            const unsigned r = vlin % G_sz;
-            iz = (int)(vlin / G_sz) - 1;
-            iy = (int)(r / G_sy) - 1;
-            ix = (int)(r % G_sy) - 1;
-        }
-        const R hh = R(p.h);
-        const R ex = (R(ix) + qx) * hh, ey = (R(iy) + qy) * hh, ez = (R(iz) + qz) * hh;
-        const unsigned long long rel = pid - p.photon_offset;
-        if (rel < p.exit_log) {
-            mcx_exit e;
-            e.fate = fate; e.nscat = nscat;
-            e.pos[0] = float(ex); e.pos[1] = float(ey); e.pos[2] = float(ez);
-            e.dir[0] = float(ux); e.dir[1] = float(uy); e.dir[2] = float(uz);
-            e.w = float(w); e.t = float(t);
-            p.exits[rel] = e;
-        }
-        if (DET && fate == MCX_FATE_ESCAPED) {
-            const float vx = float(R(ix) + qx), vy = float(R(iy) + qy), vz = float(R(iz) + qz);
-            for (int d = 0; d < p.n_det; ++d) {
-                const float4 D = s_det[d];
-                const float dx = vx - D.x, dy = vy - D.y, dz = vz - D.z;
-                if (dx * dx + dy * dy + dz * dz <= D.w) {
-                    atomicAdd(&s_stats[MCX_STAT_DETECTED], 1ull);
-                    const unsigned long long slot_i = atomicAdd(p.det_count, 1ull);
-                    if (slot_i < p.max_detected) {
+                    if (DET) {
                         if (lab < kMaxDetMedia) Lpath[lab] += float(Lcur);
-                        float *rec = p.det_buf + slot_i * (unsigned long long)p.rec_stride;
-                        rec[0] = __uint_as_float((unsigned)(pid & 0xffffffffull));
-                        rec[1] = __uint_as_float((unsigned)(pid >> 32));
-                        rec[2] = __int_as_float(d);
-                        rec[3] = __uint_as_float(nscat);
-                        rec[4] = float(w);
-                        rec[5] = float(ex); rec[6] = float(ey); rec[7] = float(ez);
-                        rec[8] = float(ux); rec[9] = float(uy); rec[10] = float(uz);
-                        rec[11] = __uint_as_float(nrr);
-                        for (int m = 1; m < p.n_media && m < kMaxDetMedia; ++m)
-                            rec[kRecBase + m - 1] = Lpath[m] * p.h;
-                    } else {
-                        atomicOr(p.status, kStatusDetOverflow);
+                        Lcur = R(0);
                     }
-                    break;
+                    lab = b;
+                    A_cur = medA(b);
+                    tpl_cur = med_tpl(b);
+                    B_cur = medB(b);
                 }
+                if (escape) state = kOver + MCX_FATE_ESCAPED;
+                else if (s <= R(0)) new_hop();        // hop used up by rounding at the face
             }
         }
-        alive = false;
     }
 
     __syncthreads();
@@ -925,9 +1004,25 @@ cudaError_t shape_for(int block, int n_media, int n_det, int tile_e, LaunchShape
     return cudaSuccess;
 }
 
-template <typename R, bool DET, int ACC, bool ST, bool BATCH = false, bool PAD = true>
-cudaError_t launch(const WalkParams &p, const LaunchShape &s, cudaStream_t st)
+// How a run's photons are shared out: all lanes and the caller's claim size, or, when there
+// are fewer photons than lanes, as few warps of each block as hold the block's share.
+WalkParams shared_out(WalkParams p, const LaunchShape &s)
 {
+    const unsigned wpb = (unsigned)s.block / 32u, grid = (unsigned)s.grid;
+    p.lanes = 32;
+    p.warps = wpb;
+    if (p.claim_static || p.n_photons >= 32ull * wpb * grid) return p;
+    const unsigned per_block = p.n_photons ? ((unsigned)p.n_photons + grid - 1u) / grid : 1u;
+    p.warps = (per_block + 31u) / 32u;
+    p.lanes = (per_block + p.warps - 1u) / p.warps;
+    p.claim_chunk = p.lanes;
+    return p;
+}
+
+template <typename R, bool DET, int ACC, bool ST, bool BATCH = false, bool PAD = true>
+cudaError_t launch(const WalkParams &params, const LaunchShape &s, cudaStream_t st)
+{
+    const WalkParams p = shared_out(params, s);
     const int tile_e = ACC == kAccCompensated
         ? p.tile_size[0] * p.tile_size[1] * p.tile_size[2] * p.tile_size[3] : 0;
     const size_t smem = SmemLayout<R>(BATCH ? 0 : p.n_media, DET ? p.n_det : 0, tile_e).total;

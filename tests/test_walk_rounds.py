@@ -1,0 +1,69 @@
+"""The walk's rounds: how a short run's photons are shared out among lanes, and the rarely
+taken path of a segment (gate changes, the time limit, the event cap, the roulette,
+near-axial directions), where each can go wrong.
+
+A run is a function of (seed, photon ids), so the sharing must not change a single photon:
+those comparisons are exact.  The rare path runs in the FP64 instantiation against the
+oracle: both follow the same decisions, up to photons whose FP64 rounding meets one of
+them (at most 1 in 1000, as in the other fixed-seed tests).
+"""
+import numpy as np
+import pytest
+
+import workloads
+from gpu_common import F32_RR, balance, f32, gpu_run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    from paper_1711_03244_gb300 import build
+    build.build()
+    import paper_1711_03244_gb300 as m
+    m.load()
+    return m
+
+
+@pytest.fixture(scope="module")
+def reference(g):
+    """600 photons with every lane of the default grid open to the first claims"""
+    return gpu_run(f32(workloads.c1()), n_photons=600, exit_log=600, seed=5)
+
+
+# 4 blocks of 64 threads: 8 warps, 256 lanes; a block's share fills one warp at 128 photons
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 127, 128, 129, 255, 256, 257, 600])
+@pytest.mark.parametrize("block,grid", [(64, 4), (32, 1), (256, 0)])
+def test_sharing_does_not_change_photons(g, reference, n, block, grid):
+    r = gpu_run(f32(workloads.c1()), n_photons=n, exit_log=600, seed=5, block_size=block, grid_size=grid)
+    assert r["stats"]["photons"] == n
+    assert np.array_equal(r["exits"][:n], reference["exits"][:n])
+    assert balance(r["tally"]) == pytest.approx(n, rel=1e-6)
+
+
+@pytest.mark.parametrize("case", ["gates", "limit", "cap", "roulette", "axial"])
+def test_rare_path_matches_oracle(g, case):
+    import oracle as orc
+    n, kw, okw = 1000, {}, {}
+    wl = f32(workloads.c1(n_photons=n).with_(labels=np.ones((16, 16, 16), dtype=np.uint8),
+                                             src_pos=(8.0, 8.0, 0.0)))
+    if case == "gates":                       # gates as long as a mean free path
+        wl = f32(wl.with_(n_gates=200, dt_ns=0.0005))
+    elif case == "limit":                     # most photons end at the limit
+        wl = f32(wl.with_(n_gates=3, dt_ns=0.02))
+    elif case == "cap":
+        kw["max_events"] = okw["max_events"] = 257
+    elif case == "roulette":
+        kw["rr_threshold"] = okw["rr_threshold"] = float(np.float32(0.7))
+        kw["rr_m"] = okw["rr_m"] = 2.0
+    else:                                     # forward scattering within 0.5 degrees of the axis
+        wl = f32(wl.with_(media=np.array([workloads.AIR, (0.01, 1.0, 0.9999, 1.37)])))
+    g64 = gpu_run(wl, exit_log=n, precision=1, **{"rr_threshold": F32_RR, **kw})
+    o = orc.run(wl, exit_cap=n, **{"rr_threshold": F32_RR, **okw})
+    same = (g64["exits"]["fate"] == o.exits["fate"]) & (g64["exits"]["nscat"] == o.exits["nscat"])
+    print(f"{case}: {same.mean():.4f} of the photons match")
+    assert same.mean() >= 0.999
+    # a deposit moves to the neighbouring gate where the two roundings of a time meet its
+    # edge: at most one photon's weight in 1000
+    d = np.abs(g64["energy"].astype(np.float64).reshape(-1) - o.energy.reshape(-1)).sum()
+    assert d <= 2e-3 * o.energy.sum()
