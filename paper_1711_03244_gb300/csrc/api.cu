@@ -617,6 +617,7 @@ mcx_status mcx_run(mcx_sim *s, const mcx_run_cfg *cfg)
         f.rr_inv_m = (float)d.rr_inv_m;
     }
     p.src_kind = s->src_kind;
+    find_hot_voxels(p, p.cd.src_pos, p.cd.src_dir, 1u, s->n_media, s->props.data(), s->h);
     p.n_photons = cfg->n_photons;
     p.photon_offset = cfg->photon_offset;
     p.seed = cfg->seed;

@@ -15,6 +15,8 @@ constexpr int kMaxDetMedia = 33;     // media rows allowed when detectors are pr
 constexpr int kMaxDet = 64;
 constexpr int kRecBase = 12;         // detected-record words before the partial paths
 constexpr int kClaimChunk = 32;      // default photon ids a warp claims per global atomic
+constexpr int kHot = 4;              // voxels of a pencil beam summed per warp
+constexpr float kHotMaxMus = 6.f;    // largest mus h at which they are
 constexpr float kC0 = 299.792458f;   // mm/ns
 
 // device status word bits
@@ -101,6 +103,10 @@ struct WalkParams {
     unsigned claim_chunk;             // photon ids a warp claims per global atomic (>= lanes)
     unsigned lanes, warps;            // lanes per warp and warps per block that take photons;
                                       // set at the launch
+    // pencil beam: the first voxels on its ray, as indices into the map's gate 0 (n_hot = 0:
+    // every deposit goes to the map)
+    int n_hot;
+    unsigned hot[kHot];
     const BatchSim *sims;             // batch: [n_sims], ordered by `first`
     int n_sims;
 };
@@ -149,6 +155,48 @@ inline void launch_plane(const double d[3], double e1[3], double e2[3])
     e2[0] = d[1] * e1[2] - d[2] * e1[1];
     e2[1] = d[2] * e1[0] - d[0] * e1[2];
     e2[2] = d[0] * e1[1] - d[1] * e1[0];
+}
+
+// The voxels that an undeflected photon of a pencil beam crosses first, for the walk to sum
+// per warp in shared memory (pos in voxel units; p's volume, strides and source kind set; pad
+// = 1 for the bordered layout).  Every photon deposits into them, and the L2 adds to one
+// address at about 3.6e8/s: that bounds a run whose photons are short.  Photons that scatter
+// often are too slow to meet it, and the test in every face step would cost them 2%, so the
+// rule asks for mus h <= 6 in every tissue (B1, mus h = 1, 1e7 photons: 27.3 -> 17.8 ms;
+// B2a, 1 and 5: 33.8 -> 29.4 ms; two spheres, 10 / 5 / 1, 2e7 photons, with them: 151.7 ->
+// 155.6 ms).  The list decides where a sum is kept, never what is added: a photon that
+// rounding or refraction takes off the ray deposits as usual.
+inline void find_hot_voxels(WalkParams &p, const double pos[3], const double dir[3], unsigned pad,
+                            uint32_t n_media, const float *props, float h)
+{
+    p.n_hot = 0;
+    if (p.src_kind != 0) return;
+    for (uint32_t m = 1; m < n_media; ++m)
+        if (!(props[4 * m + 1] * h <= kHotMaxMus)) return;
+    const int dim[3] = {p.nx, p.ny, p.nz};
+    double q[3];
+    int c[3];
+    for (int a = 0; a < 3; ++a) {
+        const float x = (float)pos[a];
+        if (!(x >= 0.f) || !(x <= (float)dim[a])) return;
+        const float f = __builtin_floorf(x);
+        c[a] = (int)f - ((x == f && dir[a] < 0) ? 1 : 0);
+        q[a] = (double)x - c[a];
+    }
+    while (p.n_hot < kHot) {
+        for (int a = 0; a < 3; ++a)
+            if (c[a] < 0 || c[a] >= dim[a]) return;
+        p.hot[p.n_hot++] = ((unsigned)c[2] + pad) * p.sz + ((unsigned)c[1] + pad) * p.sy + ((unsigned)c[0] + pad);
+        double l = 1e300;
+        int ax = 0;
+        for (int a = 0; a < 3; ++a) {
+            const double d = dir[a] > 0 ? (1.0 - q[a]) / dir[a] : (dir[a] < 0 ? -q[a] / dir[a] : 1e300);
+            if (d < l) { l = d; ax = a; }
+        }
+        for (int a = 0; a < 3; ++a) q[a] += l * dir[a];
+        c[ax] += dir[ax] > 0 ? 1 : -1;
+        q[ax] = dir[ax] > 0 ? 0.0 : 1.0;
+    }
 }
 
 // api.cu: the error text mcx_last_error(NULL) returns (per host thread)

@@ -284,6 +284,8 @@ extern "C" mcx_status mcx_run_noalloc(const uint8_t *labels_dev, uint32_t nx, ui
     c.rr_m = cfg->rr_m;
     c.rr_inv_m = cfg->rr_threshold > 0.f ? (float)(1.0 / (double)cfg->rr_m) : 0.f;
     p.src_kind = src_kind;
+    const double pos[3] = {c.src_pos[0], c.src_pos[1], c.src_pos[2]};
+    find_hot_voxels(p, pos, d, 0u, n_media, props, voxel_mm);
     p.n_photons = cfg->n_photons;
     p.photon_offset = cfg->photon_offset;
     p.seed = cfg->seed;

@@ -272,16 +272,19 @@ __device__ __forceinline__ R face_dist(R q, R inv)
 
 // ------------------------------------------------------------------------------ kernel
 // Dynamic shared memory, sized by the run's media and detector counts:
-//   double tally[8] | u64 stats[8] | MedA<R>[n_media] | MedB<R>[n_media] | R n[n_media] |
+//   double tally[8] | u64 stats[8] | double hot[8 warps][kHot], u32 hot voxel[kHot] | MedA<R>[n_media] | MedB<R>[n_media] | R n[n_media] |
 //   R tpl[n_media] | float4 det[n_det]
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
+constexpr size_t kHotBytes = 8 * kHot * sizeof(double) + kHot * sizeof(unsigned);
+
 template <typename R>
 struct SmemLayout {
-    size_t a, b, n, tpl, det, tile, total;
+    size_t hot, a, b, n, tpl, det, tile, total;
     __host__ __device__ SmemLayout(int n_media, int n_det, int tile_entries)
     {
-        a = 128;
+        hot = 128;
+        a = hot + kHotBytes;
         b = align16(a + sizeof(MedA<R>) * n_media);
         n = align16(b + sizeof(MedB<R>) * n_media);
         tpl = align16(n + sizeof(R) * n_media);
@@ -315,9 +318,12 @@ template <> __device__ __forceinline__ const RunConsts<double> &consts<double>(c
 // without per-axis bounds checks, and the per-axis voxel indices need not be carried
 // (they are recovered from the linear index when a photon ends).  Caller-owned unpadded
 // buffers (the allocation-free run) take PAD = false.
+// HOT: a pencil beam's first voxels are summed per warp in shared memory and added to the
+// map when the block ends (find_hot_voxels; FP64 accumulation, so that the regrouped sum
+// loses nothing).
 // FP32: 4 resident blocks of 256 threads per SM (64 registers; the batch instantiation too,
 // with a few spilled words for its per-lane simulation geometry)
-template <typename R, bool DET, int ACC, bool STATIC, bool BATCH, bool PAD>
+template <typename R, bool DET, int ACC, bool STATIC, bool BATCH, bool PAD, bool HOT>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1)
 walk_kernel(const WalkParams p)
 {
@@ -345,6 +351,14 @@ walk_kernel(const WalkParams p)
         for (int i = threadIdx.x; i < p.n_det; i += blockDim.x) s_det[i] = p.det[i];
     if (threadIdx.x < 8) s_tally[threadIdx.x] = 0.0;
     if (threadIdx.x < 8) s_stats[threadIdx.x] = 0ull;
+    double *s_hot = reinterpret_cast<double *>(smem_raw + L.hot);
+    unsigned *s_hot_voxel = reinterpret_cast<unsigned *>(s_hot + 8 * kHot);
+    if (HOT) {
+        for (int i = threadIdx.x; i < 8 * kHot; i += blockDim.x) s_hot[i] = 0.0;
+        // looked up in shared memory: an index that differs from lane to lane serialises
+        // reads of the parameter bank (B1: 55 ms)
+        if (threadIdx.x < kHot) s_hot_voxel[threadIdx.x] = (int)threadIdx.x < p.n_hot ? p.hot[threadIdx.x] : ~0u;
+    }
     if (ACC == kAccCompensated)
         for (int i = threadIdx.x; i < 2 * tile_e; i += blockDim.x) s_hi[i] = 0.f;
     __syncthreads();
@@ -428,8 +442,10 @@ walk_kernel(const WalkParams p)
     int axis = 0;                 // the axis of the face that ends the lane's segment
     int again = 1;                // walking lanes with which the warp goes on with segments
 
-    // a6/a12: one accumulation per (gate, voxel) run of deposits
-    auto flush = [&]() {
+    // a6/a12: one accumulation per (gate, voxel) run of deposits.  in_voxel: the run ends with
+    // a crossing into the same medium, as the first ones of a beam do
+    auto flush = [&](auto in_voxel) {
+        constexpr bool MAY_HOT = HOT && decltype(in_voxel)::value;
         if (acc != R(0)) {
             const unsigned long long idx = (unsigned long long)gate * G_nvox + vlin;
             // one fire-and-forget FP64 add into the map; for FP32 the (positive, normal: the
@@ -448,7 +464,11 @@ walk_kernel(const WalkParams p)
             if (ACC == kAccPlain) {
                 atomicAdd(G_flu + idx, float(acc));
             } else if (ACC == kAccF64) {
-                add_f64();
+                // the photon's k-th run, on the ray's k-th voxel
+                if (MAY_HOT && c_flush < (unsigned)kHot && gate == 0u && vlin == s_hot_voxel[c_flush])
+                    atomicAdd(s_hot + (threadIdx.x >> 5) * kHot + c_flush, double(acc));
+                else
+                    add_f64();
             } else {
                 // compensated: runs inside the block tile go to its shared-memory (hi, lo)
                 // pair, the rest to the FP64 map
@@ -512,7 +532,7 @@ walk_kernel(const WalkParams p)
                 // ---- photon finished: flush the deposit run, tallies, logs, detectors (a9, a12)
                 const int fate = state - kOver;
                 const unsigned nscat = nev - c_face;          // every counted segment ends in either
-                flush();
+                flush(std::false_type{});
                 const R absorbed = R(1) + gained - w;
                 const int slot = fate == MCX_FATE_ESCAPED ? MCX_TALLY_ESCAPED
                                : (fate == MCX_FATE_ROULETTE ? MCX_TALLY_RR_KILLED : MCX_TALLY_TIME);
@@ -730,7 +750,7 @@ walk_kernel(const WalkParams p)
                         state = kOver + MCX_FATE_CAPPED;
                     } else {
                         if (t >= t_next) {                // a7: the gate of this segment's start
-                            flush();
+                            flush(std::false_type{});
                             unsigned g2 = (unsigned)(t * C.inv_dt);
                             g2 = g2 > gate + 1u ? g2 : gate + 1u;
                             gate = g2 < last_gate ? g2 : last_gate;
@@ -799,7 +819,7 @@ walk_kernel(const WalkParams p)
             }
             if (b == lab) {
                 // same medium: straight into the next voxel, entering on the near face
-                flush();                              // the deposit run ends with the voxel
+                flush(std::true_type{});              // the deposit run ends with the voxel
                 const R qn = up ? R(0) : R(1);
                 qx = p0 ? qn : qx;
                 qy = p1 ? qn : qy;
@@ -853,7 +873,7 @@ walk_kernel(const WalkParams p)
                     }
                 }
                 if (enter) {
-                    flush();
+                    flush(std::false_type{});
                     if constexpr (AXES) {
                         ix = p0 ? ia : ix;
                         iy = p1 ? ia : iy;
@@ -892,6 +912,9 @@ walk_kernel(const WalkParams p)
             atomicAdd(G_flu64 + (unsigned long long)(p.tile_lo[3] + tg) * G_nvox + vl, v);
         }
     }
+    if (HOT)
+        for (int i = threadIdx.x; i < 8 * kHot; i += blockDim.x)
+            if (s_hot[i] != 0.0) atomicAdd(G_flu64 + s_hot_voxel[i % kHot], s_hot[i]);
     if (threadIdx.x < MCX_NTALLY)
         p.block_tally[(size_t)blockIdx.x * MCX_NTALLY + threadIdx.x] = s_tally[threadIdx.x];
     if (threadIdx.x < MCX_NSTAT)
@@ -985,18 +1008,18 @@ template <typename R, bool DET, int ACC, bool ST, bool BATCH = false, bool PAD =
 cudaError_t shape_for(int block, int n_media, int n_det, int tile_e, LaunchShape *shape)
 {
     const size_t smem = SmemLayout<R>(n_media, DET ? n_det : 0, tile_e).total;
-    cudaError_t e = cudaFuncSetAttribute(walk_kernel<R, DET, ACC, ST, BATCH, PAD>,
+    cudaError_t e = cudaFuncSetAttribute(walk_kernel<R, DET, ACC, ST, BATCH, PAD, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel<R, DET, ACC, ST, BATCH, PAD>,
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel<R, DET, ACC, ST, BATCH, PAD, false>,
                                                            block, smem)) != cudaSuccess)
         return e;
     cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, walk_kernel<R, DET, ACC, ST, BATCH, PAD>)) != cudaSuccess) return e;
+    if ((e = cudaFuncGetAttributes(&fa, walk_kernel<R, DET, ACC, ST, BATCH, PAD, false>)) != cudaSuccess) return e;
     shape->block = block;
     shape->blocks_per_sm = per_sm;
     shape->grid = sms * (per_sm > 0 ? per_sm : 1);
@@ -1026,7 +1049,13 @@ cudaError_t launch(const WalkParams &params, const LaunchShape &s, cudaStream_t 
     const int tile_e = ACC == kAccCompensated
         ? p.tile_size[0] * p.tile_size[1] * p.tile_size[2] * p.tile_size[3] : 0;
     const size_t smem = SmemLayout<R>(BATCH ? 0 : p.n_media, DET ? p.n_det : 0, tile_e).total;
-    walk_kernel<R, DET, ACC, ST, BATCH, PAD><<<s.grid, s.block, smem, st>>>(p);
+    if constexpr (sizeof(R) == 4 && ACC == kAccF64 && !ST && !BATCH) {
+        if (p.n_hot > 0) {
+            walk_kernel<R, DET, ACC, ST, BATCH, PAD, true><<<s.grid, s.block, smem, st>>>(p);
+            return cudaGetLastError();
+        }
+    }
+    walk_kernel<R, DET, ACC, ST, BATCH, PAD, false><<<s.grid, s.block, smem, st>>>(p);
     return cudaGetLastError();
 }
 

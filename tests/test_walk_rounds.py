@@ -67,3 +67,30 @@ def test_rare_path_matches_oracle(g, case):
     # edge: at most one photon's weight in 1000
     d = np.abs(g64["energy"].astype(np.float64).reshape(-1) - o.energy.reshape(-1)).sum()
     assert d <= 2e-3 * o.energy.sum()
+
+
+# beams whose first voxels are summed per warp, against the same run with every deposit sent
+# to the map (an unused medium that scatters strongly turns the sums off): the FP64 sums are
+# regrouped, so they agree to FP64 rounding over 2e4 additions
+@pytest.mark.parametrize("block", [32, 256])
+@pytest.mark.parametrize("name,pos,direction,reflect,gates", [
+    ("z", (30.0, 30.0, 0.0), (0.0, 0.0, 1.0), 0, 1),
+    ("z_reflect_gates", (30.0, 30.0, 0.0), (0.0, 0.0, 1.0), 1, 7),
+    ("inside_down", (10.5, 20.25, 33.75), (0.0, 0.0, -1.0), 1, 1),
+    ("x_from_far_face", (60.0, 12.0, 7.5), (-1.0, 0.0, 0.0), 1, 2),
+    ("oblique", (0.0, 17.3, 4.2), (0.6, 0.64, 0.48), 1, 1),
+    ("corner", (0.0, 0.0, 0.0), (1.0, 1.0, 1.0), 1, 1),
+    ("last_voxel", (59.5, 59.5, 59.5), (0.0, 0.0, 1.0), 1, 1),
+])
+@pytest.mark.parametrize("variant", ["B1", "B2A"])
+def test_beam_voxel_sums(g, variant, name, pos, direction, reflect, gates, block):
+    wl = f32(workloads.paper_b(variant, n_photons=20000).with_(src_pos=pos, src_dir=direction))
+    maps, stats = [], []
+    for media in (wl.media, np.concatenate([wl.media, [[0.01, 100.0, 0.9, 1.37]]])):
+        with g.Simulation.from_workload(wl.with_(media=media)) as sim:
+            sim.run(20000, n_gates=gates, dt_ns=0.2, seed=3, reflect=reflect, block_size=block)
+            maps.append(sim.fluence64())
+            stats.append(sim.stats())
+    assert stats[0] == stats[1]
+    assert np.array_equal(maps[0] > 0, maps[1] > 0)
+    assert np.allclose(maps[0], maps[1], rtol=20000 * 2.0 ** -53, atol=0)
