@@ -8,9 +8,10 @@
 // fallback.  (This extends the method; the paper has no counterpart.)
 //
 // Layout: activations are BF16, [batch][z][y][x][channels] (channels innermost);
-// convolution weights are BF16 [27 taps][Cout][Cin] for the forward pass and
-// [27 taps][Cin][Cout] with flipped taps for the input gradient; FP32 master weights,
-// gradients and Adam moments live beside them.
+// convolution weights are BF16, packed as the kernels' shared-memory operands
+// (packed_weight), once for the forward pass and once with flipped taps and exchanged
+// channels for the input gradient; FP32 master weights ([27 taps][Cout][Cin]), gradients and
+// Adam moments live beside them.
 //
 // Network (residual: output = input + head):
 //   e1: conv(1->16), conv(16->16)      at D        skip s1
@@ -71,10 +72,8 @@ struct Vol {
 // memory as consecutive 32-byte rows in q order, swizzled by the TMA unit in the 32-byte
 // pattern -- the K-major SWIZZLE_32B operand layout (one row holds one MMA's K = 16;
 // 8-row groups 256 B apart), so a one-row shift of the operand is a 32-byte shift of its
-// start address (the swizzle follows absolute shared addresses).  Two 16-channel groups
-// per 32-byte row halve the TMA rows of the earlier 8-channel boxes.  conv3d_fwd_ws stages
-// 8-channel boxes of 16-byte rows in the no-swizzle layout
-// (8-row core matrices 128 B apart; chunks one leading-dimension offset apart).  A tile
+// start address (the swizzle follows absolute shared addresses).  16 channels per 32-byte
+// row halve the TMA rows of 8-channel boxes in the no-swizzle layout.  A tile
 // takes 3 windows (one per plane); each feeds 9 taps x cin/16 tcgen05.mma instructions
 // (K = 16, N = COUT).
 //
@@ -84,7 +83,8 @@ struct Vol {
 // "acc full"; warps 2-5 read the accumulator out (tcgen05.ld; warp w reads TMEM lanes
 // 32 (w mod 4) ...), arrive on "acc empty", and store bias + ReLU in BF16 for the valid
 // rows.  Several TMEM accumulators let a tile's read-out overlap the next tiles' MMAs.
-// The layer's weights stay resident in shared memory when they fit (one TMA load each).
+// The layer's weights stay resident in shared memory (one bulk copy; larger ones take
+// conv3d_fwd_ws).
 // With cout = 16 the three tiles a window feeds sit in consecutive accumulators and take
 // one MMA of N = 48 per (dy, dx) tap and K step (two where the accumulator ring wraps), so
 // the window's A rows are read from shared memory once instead of three times.
@@ -140,6 +140,19 @@ __host__ __device__ constexpr bool tc_wall(int cin, int cout) { return 27 * cin 
 // cout 32 the same scheme measured slower (four accumulators: the MMA thread waits for
 // read-outs, since a tile completes only with the whole window's MMAs)
 __host__ __device__ constexpr bool tc_merge(int cin, int cout) { return tc_wall(cin, cout) && cout == 16; }
+// Position of weight (tap, co, ci) in the packed layout that the kernels copy to shared memory
+// as it stands: rows of 8 input channels (16 B, the K-major no-swizzle operand layout), the
+// cout rows of a tap and 8-channel chunk together; merged layers keep, per (dy, dx) tap and
+// chunk, the rows of dz = +1, 0, -1 one after another.  One bulk copy then brings a layer's
+// (or a plane's) weights, where boxes of 16-byte rows from a [tap][cout][cin] array took 3 to
+// 11 us in every CTA (0.6 rows per clock and SM).
+__host__ __device__ inline size_t packed_weight(int tap, int co, int ci, int cin, int cout)
+{
+    const int c = ci / 8, e = ci % 8;
+    if (tc_merge(cin, cout))
+        return ((size_t)((tap % 9 * (cin / 8) + c) * 3 + (2 - tap / 9)) * cout + co) * 8 + e;
+    return ((size_t)(tap * (cin / 8) + c) * cout + co) * 8 + e;
+}
 // TMEM columns per accumulator and accumulators per CTA (the launch counts their product
 // against an SM's 512 columns when it sizes the grid)
 __host__ __device__ constexpr int tc_ncol(int cin, int cout)
@@ -148,22 +161,20 @@ __host__ __device__ constexpr int tc_ncol(int cin, int cout)
 }
 __host__ __device__ constexpr int tc_nslot(int cin, int cout)
 {
-    return tc_merge(cin, cout) ? 8 : (tc_wall(cin, cout) ? 4 : 2);
+    return tc_merge(cin, cout) ? 8 : 4;
 }
 // lines of a window: the tile's rows q0 - 1 - PW .. q0 + 128 + PW
 __host__ __device__ constexpr int tc_lines(int w) { return (kTcRows + 2 + w + 1) / (w + 2) + 3; }
-// one 8-channel chunk of a window: L lines x PW rows of 16 B, padded to 128 B
-__host__ __device__ constexpr int tc_lbo_a(int w) { return ((tc_lines(w) * (w + 2) * 16 + 127) / 128) * 128; }
 // one 16-channel group of a window: L lines x PW rows of 32 B, swizzled in 256-byte atoms
 // (SWIZZLE_32B), padded to 1 KiB so that every group starts on a swizzle-atom boundary
 __host__ __device__ constexpr int tc_gbytes(int w) { return ((tc_lines(w) * (w + 2) * 32 + 1023) / 1024) * 1024; }
-__host__ __device__ constexpr int tc_stage_bytes(int cin, int cout, int w)
+__host__ __device__ constexpr int tc_stage_bytes(int cin, int w)
 {
-    return (cin / 16) * tc_gbytes(w) + (tc_wall(cin, cout) ? 0 : ((9 * cout * cin * 2 + 1023) / 1024) * 1024);
+    return (cin / 16) * tc_gbytes(w);
 }
 __host__ __device__ constexpr int tc_smem_bytes(int cin, int cout, int w, int ns)
 {
-    return 1024 + kTcFwdHeader + (tc_wall(cin, cout) ? 27 * cout * cin * 2 : 0) + 1024 + ns * tc_stage_bytes(cin, cout, w);
+    return 1024 + kTcFwdHeader + 27 * cout * cin * 2 + 1024 + ns * tc_stage_bytes(cin, w);
 }
 // shared-memory descriptor of a K-major operand in the 32-byte swizzle (layout type 6):
 // rows of 32 B (K = 16 BF16, one MMA's K), 8-row groups 256 B apart (SBO); the leading
@@ -227,11 +238,11 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map
                    "r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar)
+// contiguous copy to shared memory; addresses and size multiples of 16 bytes
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
 {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                 " [%0], [%1, {%2, %3}], [%4];\n"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                 ::"r"(dst), "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(bar) : "memory");
 }
 
 __device__ __forceinline__ void tc_commit(uint32_t bar)
@@ -241,12 +252,12 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kTcThreads)
-conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw,
+conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ W,
               const float *__restrict__ bias, Vol v, int relu, bf16 *__restrict__ Y, unsigned *err, int ns,
               int zc)
 {
     constexpr int cin = CIN;
-    constexpr bool WALL = tc_wall(CIN, COUT);
+    static_assert(tc_wall(CIN, COUT), "larger weights take conv3d_fwd_ws");
     constexpr bool MERGE = tc_merge(CIN, COUT);
     constexpr int NCOL = tc_ncol(CIN, COUT);                           // TMEM columns per accumulator
     constexpr int NSLOT = tc_nslot(CIN, COUT);                         // accumulators per CTA
@@ -260,10 +271,9 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem_raw + (base + 320 - smem_u32(smem_raw)));
     const int wtap = COUT * cin * 2, lbo_b = COUT * 16;
     const int PW = v.w + 2, L = tc_lines(v.w), lbo_a = tc_gbytes(v.w);
-    const int a_bytes = (cin / 16) * lbo_a;
     const uint32_t wres = base + kTcFwdHeader;
-    const uint32_t ring = (wres + (WALL ? 27 * wtap : 0) + 1023u) & ~1023u;
-    const int stage_bytes = tc_stage_bytes(CIN, COUT, v.w);
+    const uint32_t ring = (wres + 27 * wtap + 1023u) & ~1023u;
+    const int stage_bytes = tc_stage_bytes(CIN, v.w);
     // merged weights: per (dy, dx) tap tt and 8-channel chunk c, the rows of dz = +1, 0, -1
     // (cout each, 16 B per row) one after another, so the tiles w - 1, w, w + 1 that a
     // window of plane w feeds are consecutive N rows; chunks LBOM bytes apart
@@ -311,18 +321,11 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
     if (tid == 0) {
         // ------------------------------------------------------------ producer (TMA)
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
-        asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmw)) : "memory");
-        if (WALL && my_units) {
+        if (my_units) {
             mbar_expect_tx(wbar, 27 * wtap);
-            for (int tap = 0; tap < 27; ++tap)
-                for (int c = 0; c < cin / 8; ++c) {
-                    const int tt = tap % 9, dzi = 2 - tap / 9;    // dzi = 1 - dz
-                    const uint32_t dst = MERGE ? wres + tt * 3 * wtap + c * LBOM + dzi * COUT * 16
-                                               : wres + tap * wtap + c * lbo_b;
-                    tma_load_2d(dst, &tmw, 8 * c, tap * COUT, wbar);
-                }
+            bulk_load(wres, W, 27 * wtap, wbar);
         }
-        const uint32_t tx = (cin / 16) * (L * PW * 32) + (WALL ? 0 : 9 * wtap);
+        const uint32_t tx = (cin / 16) * (L * PW * 32);
         int b = 0, use = 0;
         for (int uj = 0; uj < my_units && ok; ++uj) {
             const Unit U = unit_of(uj);
@@ -334,10 +337,6 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
                 mbar_expect_tx(fb, tx);
                 for (int c = 0; c < cin / 16; ++c)
                     tma_load_5d(st + c * lbo_a, &tmx, 16 * c, -1, fl, U.z0 - 1 + j, U.b, fb);
-                if (!WALL)                                       // one tile per unit: dz = j - 1
-                    for (int tt = 0; tt < 9; ++tt)
-                        for (int c = 0; c < cin / 8; ++c)
-                            tma_load_2d(st + a_bytes + tt * wtap + c * lbo_b, &tmw, 8 * c, (9 * j + tt) * COUT, fb);
                 if (++b == ns) { b = 0; ++use; }
             }
         }
@@ -346,11 +345,11 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
             const int issued = use + (bb < b ? 1 : 0);       // fills of buffer bb
             if (issued > 0) ok &= mbar_wait(full0 + 8 * bb, (uint32_t)((issued - 1) & 1));
         }
-        if (WALL && my_units) ok &= mbar_wait(wbar, 0);
+        if (my_units) ok &= mbar_wait(wbar, 0);
     } else if (tid == 32) {
         // ------------------------------------------------------------ MMA issuer
-        if (WALL && my_units) ok &= mbar_wait(wbar, 0);
-        const uint64_t bdesc0 = umma_desc(WALL ? wres : ring + a_bytes, lbo_b, 128);
+        if (my_units) ok &= mbar_wait(wbar, 0);
+        const uint64_t bdesc0 = umma_desc(wres, lbo_b, 128);
         int toff[9];                                            // row offset of each (dy, dx) tap
 #pragma unroll
         for (int tt = 0; tt < 9; ++tt) toff[tt] = (tt / 3 - 1) * PW + (tt % 3 - 1);
@@ -412,8 +411,7 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
                         if (dz == -1 && T >= NSLOT)                 // the slot's previous tile is read out
                             ok &= mbar_wait(acce0 + 8 * slot, (uint32_t)((T / NSLOT - 1) & 1));
                         if (!ok) break;
-                        const uint64_t bbase = WALL ? bdesc0 + (uint64_t)((9 * (dz + 1) * wtap) >> 4)
-                                                    : bdesc0 + (uint64_t)((b * stage_bytes) >> 4);
+                        const uint64_t bbase = bdesc0 + (uint64_t)((9 * (dz + 1) * wtap) >> 4);
                         const uint32_t d = tmem + slot * NCOL;
 #pragma unroll
                         for (int tt = 0; tt < 9; ++tt)              // tt = 3 (dy + 1) + (dx + 1)
@@ -496,9 +494,10 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
 // plane's 9 taps of weights are loaded once (one buffer, refilled when the previous
 // plane's MMAs have completed), then each tile's window of that plane streams through
 // the ring.  Weights then cross L2 once per unit and plane instead of once per tile and
-// plane.  Tiles, windows, operand layouts and the bounded waits are those of
-// conv3d_fwd_tc.
-constexpr int kWsHeader = 512;
+// plane.  A small volume's units hold fewer tiles (tu), so that they reach every SM.
+// Tiles, windows, operand layouts and the bounded waits are those of conv3d_fwd_tc; a
+// seventh warp loads the weights.
+constexpr int kWsHeader = 512, kWsThreads = kTcThreads + 32;    // warp 6 loads the weights
 
 __host__ __device__ constexpr int ws_tiles_per_unit(int cout)
 {
@@ -506,7 +505,7 @@ __host__ __device__ constexpr int ws_tiles_per_unit(int cout)
 }
 __host__ __device__ constexpr int ws_smem_bytes(int cin, int cout, int w, int ns)
 {
-    return 1024 + kWsHeader + 9 * cout * cin * 2 + ns * (cin / 8) * tc_lbo_a(w);
+    return 1024 + kWsHeader + 9 * cout * cin * 2 + 1024 + ns * (cin / 16) * tc_gbytes(w);
 }
 __host__ __device__ constexpr int ws_stages(int cin, int cout, int w)
 {
@@ -516,9 +515,10 @@ __host__ __device__ constexpr int ws_stages(int cin, int cout, int w)
 }
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kTcThreads)
-conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw,
-              const float *__restrict__ bias, Vol v, int relu, bf16 *__restrict__ Y, unsigned *err, int ns)
+__global__ void __launch_bounds__(kWsThreads)
+conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ W,
+              const float *__restrict__ bias, Vol v, int relu, bf16 *__restrict__ Y, unsigned *err, int ns,
+              int tu)
 {
     constexpr int NCOL = COUT <= 32 ? 32 : (COUT <= 64 ? 64 : 128);   // TMEM columns per accumulator
     constexpr int TU = ws_tiles_per_unit(COUT);
@@ -526,19 +526,19 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;      // 1 KiB aligned
     // header: full[ns] at 0, empty[ns] at 64, acc full[2 TU] at 128, acc empty[2 TU] at 256,
-    // weights full at 384, weights empty at 392, MMA drain at 400, TMEM address at 448
+    // weights full[3] at 384, weights empty[3] at 408, MMA drain at 432, TMEM address at 448
     const uint32_t full0 = base, empty0 = base + 64, accf0 = base + 128, acce0 = base + 256;
-    const uint32_t wfull = base + 384, wempty = base + 392, drain = base + 400;
+    const uint32_t wfull = base + 384, wempty = base + 408, drain = base + 432;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem_raw + (base + 448 - smem_u32(smem_raw)));
     const int wtap = COUT * CIN * 2, lbo_b = COUT * 16;
-    const int PW = v.w + 2, L = tc_lines(v.w), lbo_a = tc_lbo_a(v.w);
-    const int a_bytes = (CIN / 8) * lbo_a;
+    const int PW = v.w + 2, L = tc_lines(v.w), lbo_a = tc_gbytes(v.w);
+    const int a_bytes = (CIN / 16) * lbo_a;
     const uint32_t wbuf = base + kWsHeader;                // one plane's 9 taps
-    const uint32_t ring = wbuf + 9 * wtap;
+    const uint32_t ring = (wbuf + 9 * wtap + 1023u) & ~1023u;
     const int tid = threadIdx.x, warp = tid >> 5;
     const int tiles_plane = (v.h * PW + kTcRows - 1) / kTcRows;
     const int n_tiles = v.n * v.d * tiles_plane;
-    const int n_units = (n_tiles + TU - 1) / TU;
+    const int n_units = (n_tiles + tu - 1) / tu;
     const int my_units = n_units > (int)blockIdx.x ? (n_units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     struct Tl { int b, z, q0; };
     auto tile_at = [&](int tile) {
@@ -547,8 +547,8 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
     };
     auto unit_tiles = [&](int uj, int &t0, int &nt) {
         const int u = (int)blockIdx.x + uj * (int)gridDim.x;
-        t0 = u * TU;
-        nt = min(TU, n_tiles - t0);
+        t0 = u * tu;
+        nt = min(tu, n_tiles - t0);
     };
     auto first_line = [&](int q0) { return (q0 >= 1 ? (q0 - 1) / PW : -1) - 1; };
 
@@ -566,8 +566,10 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
             mbar_init(accf0 + 8 * a, 1);
             mbar_init(acce0 + 8 * a, 4 * 32);
         }
-        mbar_init(wfull, 1);
-        mbar_init(wempty, 1);
+        for (int r = 0; r < 3; ++r) {
+            mbar_init(wfull + 8 * r, 1);
+            mbar_init(wempty + 8 * r, 1);
+        }
         mbar_init(drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -576,32 +578,25 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
     tc_fence_after();
     const uint32_t tmem = *tslot;
     bool ok = true;
+    int wloads = 0;                                          // planes of weights asked for
 
     if (tid == 0) {
         // ------------------------------------------------------------ producer (TMA)
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
-        asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmw)) : "memory");
-        const uint32_t tx = (CIN / 8) * (L * PW * 16);
-        int b = 0, use = 0, wpass = 0;
+        const uint32_t tx = (CIN / 16) * (L * PW * 32);
+        int b = 0, use = 0;
         for (int uj = 0; uj < my_units && ok; ++uj) {
             int t0, nt;
             unit_tiles(uj, t0, nt);
             for (int g = 0; g < 3 && ok; ++g) {               // plane z + g - 1
-                if (wpass > 0) ok &= mbar_wait(wempty, (uint32_t)((wpass - 1) & 1));
-                if (!ok) break;
-                mbar_expect_tx(wfull, 9 * wtap);
-                for (int tt = 0; tt < 9; ++tt)
-                    for (int c = 0; c < CIN / 8; ++c)
-                        tma_load_2d(wbuf + tt * wtap + c * lbo_b, &tmw, 8 * c, (9 * g + tt) * COUT, wfull);
-                ++wpass;
                 for (int t = 0; t < nt && ok; ++t) {
                     if (use > 0) ok &= mbar_wait(empty0 + 8 * b, (uint32_t)((use - 1) & 1));
                     if (!ok) break;
                     const Tl T = tile_at(t0 + t);
                     const uint32_t st = ring + b * a_bytes, fb = full0 + 8 * b;
                     mbar_expect_tx(fb, tx);
-                    for (int c = 0; c < CIN / 8; ++c)
-                        tma_load_5d(st + c * lbo_a, &tmx, 8 * c, -1, first_line(T.q0), T.z + g - 1, T.b, fb);
+                    for (int c = 0; c < CIN / 16; ++c)
+                        tma_load_5d(st + c * lbo_a, &tmx, 16 * c, -1, first_line(T.q0), T.z + g - 1, T.b, fb);
                     if (++b == ns) { b = 0; ++use; }
                 }
             }
@@ -610,10 +605,23 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
             const int issued = use + (bb < b ? 1 : 0);
             if (issued > 0) ok &= mbar_wait(full0 + 8 * bb, (uint32_t)((issued - 1) & 1));
         }
-        if (wpass > 0) ok &= mbar_wait(wfull, (uint32_t)((wpass - 1) & 1));
+    } else if (tid == kTcThreads) {
+        // ------------------------------------------------------------ producer (weights)
+        // a plane's weights in three groups of taps (dy), each refilled once the previous
+        // plane's last tile is done with it: the refill overlaps the other groups' MMAs
+        const int passes = 3 * my_units;
+        for (int q = 0; q < passes && ok; ++q)
+            for (int r = 0; r < 3 && ok; ++r) {
+                if (q > 0) ok &= mbar_wait(wempty + 8 * r, (uint32_t)((q - 1) & 1));
+                if (!ok) break;
+                mbar_expect_tx(wfull + 8 * r, 3 * wtap);
+                bulk_load(wbuf + 3 * r * wtap, W + (size_t)(9 * (q % 3) + 3 * r) * COUT * CIN, 3 * wtap, wfull + 8 * r);
+                wloads = q + 1;
+            }
+        for (int r = 0; r < 3; ++r)                           // every load has landed
+            if (wloads > 0) ok &= mbar_wait(wfull + 8 * r, (uint32_t)((wloads - 1) & 1));
     } else if (tid == 32) {
         // ------------------------------------------------------------ MMA issuer
-        const uint64_t adesc0 = umma_desc(ring, lbo_a, 128);
         const uint64_t bdesc0 = umma_desc(wbuf, lbo_b, 128);
         int toff[9];
 #pragma unroll
@@ -624,8 +632,6 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
             unit_tiles(uj, t0, nt);
             const int set = uj & 1;
             for (int g = 0; g < 3 && ok; ++g) {
-                ok &= mbar_wait(wfull, (uint32_t)(wpass & 1));
-                if (!ok) break;
                 for (int t = 0; t < nt && ok; ++t) {
                     const int slot = set * TU + t;
                     if (g == 0 && uj >= 2)                      // the slot's previous tile is read out
@@ -635,24 +641,31 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
                     tc_fence_after();
                     const Tl T = tile_at(t0 + t);
                     const int off = T.q0 - first_line(T.q0) * PW;
-                    const uint64_t abase = adesc0 + (uint64_t)((b * a_bytes + off * 16) >> 4);
+                    const uint32_t abase = ring + (uint32_t)(b * a_bytes + off * 32);
                     const uint32_t d = tmem + slot * NCOL;
 #pragma unroll
-                    for (int tt = 0; tt < 9; ++tt)
+                    for (int tt = 0; tt < 9; ++tt) {
+                        if (tt % 3 == 0 && t == 0) {             // this plane's weights of the group
+                            ok &= mbar_wait(wfull + 8 * (tt / 3), (uint32_t)(wpass & 1));
+                            tc_fence_after();
+                        }
+                        if (!ok) break;
 #pragma unroll
                         for (int kk = 0; kk < CIN / 16; ++kk) {
-                            const uint64_t ad = abase + (uint64_t)(int64_t)((toff[tt] * 16 + 2 * kk * lbo_a) >> 4);
+                            const uint64_t ad = sw32_desc(abase + (uint32_t)(toff[tt] * 32 + kk * lbo_a));
                             const uint64_t bd = bdesc0 + (uint64_t)((tt * wtap + 2 * kk * lbo_b) >> 4);
                             const uint32_t accum = (g == 0 && tt == 0 && kk == 0) ? 0u : 1u;
                             asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                                          " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
                                          ::"r"(d), "l"(ad), "l"(bd), "r"(IDESC), "r"(accum) : "memory");
                         }
+                        if (tt % 3 == 2 && t == nt - 1) tc_commit(wempty + 8 * (tt / 3));
+                    }
+                    if (!ok) break;
                     tc_commit(empty0 + 8 * b);
                     if (g == 2) tc_commit(accf0 + 8 * slot);    // tile t of the unit is complete
                     if (++b == ns) { b = 0; ++use; }
                 }
-                tc_commit(wempty);                              // this plane's weights are free
                 ++wpass;
             }
         }
@@ -660,7 +673,7 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
         // a wait above gave up (the epilogue then no longer waits for the accumulators)
         tc_commit(drain);
         ok &= mbar_wait(drain, 0);
-    } else if (warp >= 2) {
+    } else if (warp >= 2 && warp < 6) {
         // ------------------------------------------------------------ epilogue
         const int quarter = warp & 3, r = quarter * 32 + (tid & 31);
         for (int uj = 0; uj < my_units && ok; ++uj) {
@@ -1054,7 +1067,7 @@ conv_in_fwd(const float *__restrict__ x, const bf16 *__restrict__ W, const float
     __shared__ float4 sw[27][4];                  // W[tap][co][ci = 0], 4 channels per float4
     __shared__ float sb[16];
     for (int i = threadIdx.x; i < 27 * 16; i += blockDim.x)
-        reinterpret_cast<float *>(sw)[i] = __bfloat162float(W[(size_t)i * 16]);   // [27][16][16]
+        reinterpret_cast<float *>(sw)[i] = __bfloat162float(W[packed_weight(i / 16, i % 16, 0, 16, 16)]);
     if (threadIdx.x < 16) sb[threadIdx.x] = bias ? bias[threadIdx.x] : 0.f;
     __syncthreads();
     const int nquad = (int)(v.pos() / 4), wq = v.w / 4;
@@ -1266,8 +1279,7 @@ __global__ void head_bwd(const bf16 *Y, const float *out, const float *target, c
     }
 }
 
-// Adam on the FP32 master weights; refreshes the BF16 forward copy [tap][co][ci] and the
-// input-gradient copy [26 - tap][ci][co] of convolution weights
+// Adam on the FP32 master weights
 __global__ void adam_step(float *w, const float *gr, float *m, float *v, long long n, float lr,
                           float b1, float b2, float c1, float c2, float eps)
 {
@@ -1282,6 +1294,8 @@ __global__ void adam_step(float *w, const float *gr, float *m, float *v, long lo
     }
 }
 
+// the BF16 copies of a convolution's weights, packed: [tap][co][ci] for the forward pass and
+// [26 - tap][ci][co] for the input gradient
 __global__ void refresh_conv_bf16(const float *w, int cin, int cout, bf16 *wf, bf16 *wb)
 {
     const long long n = 27LL * cin * cout, st = (long long)gridDim.x * blockDim.x;
@@ -1290,8 +1304,8 @@ __global__ void refresh_conv_bf16(const float *w, int cin, int cout, bf16 *wf, b
         const int co = (int)((i / cin) % cout);
         const int tap = (int)(i / ((long long)cin * cout));
         const bf16 b = __float2bfloat16(w[i]);
-        wf[i] = b;
-        wb[((size_t)(26 - tap) * cin + ci) * cout + co] = b;
+        wf[packed_weight(tap, co, ci, cin, cout)] = b;
+        wb[packed_weight(26 - tap, ci, co, cout, cin)] = b;
     }
 }
 
@@ -1382,22 +1396,14 @@ cudaError_t launch_tc_t(const bf16 *X, const bf16 *W, const float *bias, Vol v, 
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
     // activations [n][d][h][w][cin] as a 5-D tensor, innermost first
-    CUtensorMap mx, mw;
+    CUtensorMap mx;
     const cuuint64_t xdim[5] = {(cuuint64_t)cin, (cuuint64_t)v.w, (cuuint64_t)v.h, (cuuint64_t)v.d, (cuuint64_t)v.n};
     const cuuint64_t xstr[4] = {(cuuint64_t)cin * 2, (cuuint64_t)v.w * cin * 2, (cuuint64_t)v.h * v.w * cin * 2,
                                 (cuuint64_t)v.d * v.h * v.w * cin * 2};
-    const cuuint32_t xbox[5] = {8, (cuuint32_t)(v.w + 2), (cuuint32_t)tc_lines(v.w), 1, 1};
+    const cuuint32_t xbox[5] = {16, (cuuint32_t)(v.w + 2), (cuuint32_t)tc_lines(v.w), 1, 1};
     const cuuint32_t one[5] = {1, 1, 1, 1, 1};
     if (enc(&mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(X), xdim, xstr, xbox, one,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    // weights [27 * cout][cin]
-    const cuuint64_t wdim[2] = {(cuuint64_t)cin, (cuuint64_t)27 * COUT};
-    const cuuint64_t wstr[1] = {(cuuint64_t)cin * 2};
-    const cuuint32_t wbox[2] = {8, (cuuint32_t)COUT};
-    if (enc(&mw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(W), wdim, wstr, wbox, one,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     if constexpr (!tc_wall(CIN, COUT)) {
@@ -1413,45 +1419,53 @@ cudaError_t launch_tc_t(const bf16 *X, const bf16 *W, const float *bias, Vol v, 
         if ((we = cudaDeviceGetAttribute(&wsms, cudaDevAttrMultiProcessorCount, wdev)) != cudaSuccess) return we;
         const long long wtiles = (long long)v.n * v.d * ((v.h * (v.w + 2) + kTcRows - 1) / kTcRows);
         if (wtiles * 3 >= (1LL << 31)) return cudaErrorInvalidValue;
-        const long long wunits = (wtiles + ws_tiles_per_unit(COUT) - 1) / ws_tiles_per_unit(COUT);
+        // tiles per unit: the busiest CTA's tiles, plus one tile's time for each unit's
+        // three loads of weights, at their fewest
+        int tu = 1;
+        long long best = 1LL << 62;
+        for (int t = ws_tiles_per_unit(COUT); t >= 1; --t) {
+            const long long rounds = ((wtiles + t - 1) / t + wsms - 1) / wsms;
+            if (rounds * (t + 1) < best) { best = rounds * (t + 1); tu = t; }
+        }
+        const long long wunits = (wtiles + tu - 1) / tu;
         const unsigned wblocks = (unsigned)std::max<long long>(1, std::min<long long>(wunits, wsms));
-        conv3d_fwd_ws<CIN, COUT><<<wblocks, kTcThreads, wsmem, st>>>(mx, mw, bias, v, relu, Y, err, wns);
+        conv3d_fwd_ws<CIN, COUT><<<wblocks, kWsThreads, wsmem, st>>>(mx, W, bias, v, relu, Y, err, wns, tu);
+        return cudaGetLastError();
+    } else {
+        const int ns = tc_stages(cin, COUT, v.w);
+        if (ns < 2) return cudaErrorInvalidValue;                   // the volume is too wide
+        const int smem = tc_smem_bytes(cin, COUT, v.w, ns);
+        cudaError_t e = cudaFuncSetAttribute(conv3d_fwd_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        // resident CTAs per SM: shared memory (1 KiB per CTA reserved by the system), tensor
+        // memory (512 columns, NSLOT accumulators per CTA), threads
+        int dev = 0, sms = 0, smem_sm = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess)
+            return e;
+        const int per_sm = std::max(1, std::min({smem_sm / (smem + 1024), 512 / (tc_nslot(CIN, COUT) * tc_ncol(CIN, COUT)),
+                                                 2048 / kTcThreads}));
+        const long long tiles_plane = (v.h * (v.w + 2) + kTcRows - 1) / kTcRows;
+        if ((long long)v.n * v.d * tiles_plane * 3 >= (1LL << 31)) return cudaErrorInvalidValue;
+        // column depth z (of 16, 8, 4, 2, 1): a unit takes z + 2 windows.  The time is the busiest
+        // SM's windows, or the busiest CTA's at kAlone times the cost, whichever is longer: a
+        // CTA alone on its SM takes that much longer for a window than a full SM's share
+        constexpr double kAlone = 2.5;
+        int zc = 1;
+        double best = 1e300;
+        for (int z = 16; z >= 1; z /= 2) {
+            const int zz = std::min(z, v.d);
+            const long long u = (long long)v.n * ((v.d + zz - 1) / zz) * tiles_plane;
+            const long long rounds = (u + (long long)sms * per_sm - 1) / ((long long)sms * per_sm);
+            const double cost = (zz + 2) * std::max((double)((u + sms - 1) / sms), kAlone * (double)rounds);
+            if (cost < best) { best = cost; zc = zz; }
+        }
+        const long long units = (long long)v.n * ((v.d + zc - 1) / zc) * tiles_plane;
+        const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>(units, (long long)sms * per_sm));
+        conv3d_fwd_tc<CIN, COUT><<<blocks, kTcThreads, smem, st>>>(mx, W, bias, v, relu, Y, err, ns, zc);
         return cudaGetLastError();
     }
-    const cuuint32_t xbox32[5] = {16, (cuuint32_t)(v.w + 2), (cuuint32_t)tc_lines(v.w), 1, 1};
-    if (enc(&mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(X), xdim, xstr, xbox32, one,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    const int ns = tc_stages(cin, COUT, v.w);
-    if (ns < 2) return cudaErrorInvalidValue;                   // the volume is too wide
-    const int smem = tc_smem_bytes(cin, COUT, v.w, ns);
-    cudaError_t e = cudaFuncSetAttribute(conv3d_fwd_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    // resident CTAs per SM: shared memory (1 KiB per CTA reserved by the system), tensor
-    // memory (512 columns, NSLOT accumulators per CTA), threads
-    int dev = 0, sms = 0, smem_sm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess)
-        return e;
-    const int per_sm = std::max(1, std::min({smem_sm / (smem + 1024), 512 / (tc_nslot(CIN, COUT) * tc_ncol(CIN, COUT)),
-                                             2048 / kTcThreads}));
-    const long long tiles_plane = (v.h * (v.w + 2) + kTcRows - 1) / kTcRows;
-    if ((long long)v.n * v.d * tiles_plane * 3 >= (1LL << 31)) return cudaErrorInvalidValue;
-    // column depth: the deepest of 16, 8, 4, 2 that still leaves 3 units per resident CTA
-    // (a window then serves up to 3 tiles); on volumes too small for that, min(16, d);
-    // 1 without resident weights
-    int zc = 1;
-    if (tc_wall(CIN, COUT)) {
-        zc = std::min(16, v.d);
-        for (int z = 16; z >= 2; z /= 2)
-            if ((long long)v.n * ((v.d + z - 1) / z) * tiles_plane >= 3LL * sms * per_sm) { zc = z; break; }
-    }
-    const long long units = (long long)v.n * ((v.d + zc - 1) / zc) * tiles_plane;
-    const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>(units, (long long)sms * per_sm));
-    conv3d_fwd_tc<CIN, COUT><<<blocks, kTcThreads, smem, st>>>(mx, mw, bias, v, relu, Y, err, ns, zc);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_fwd_tc(const bf16 *X, int cin, const bf16 *W, const float *bias, Vol v, int cout,
@@ -1981,10 +1995,10 @@ mcx_status mcx_debug_conv3d(int32_t kind, int32_t n, int32_t dd, int32_t hh, int
     const long long P = v.pos();
     if (kind == 0 && cin == 1) {
         // the direct input layer: FP32 input, weights [27][16][1] placed at ci = 0 of the
-        // network's [27][16][16] layout
+        // network's 16 x 16 channels
         if (cout != 16 || P * 96 >= (1LL << 31)) return dn_fail(nullptr, MCX_E_ARG, "bad arguments");
         std::vector<bf16> hw16(27 * 16 * 16, __float2bfloat16(0.f));
-        for (int i = 0; i < 27 * 16; ++i) hw16[(size_t)i * 16] = __float2bfloat16(w[i]);
+        for (int i = 0; i < 27 * 16; ++i) hw16[packed_weight(i / 16, i % 16, 0, 16, 16)] = __float2bfloat16(w[i]);
         DBuf bx, bw, bb, by;
         cudaError_t e = bx.alloc(P * 4);
         if (e == cudaSuccess) e = cudaMemcpy(bx.p, x, P * 4, cudaMemcpyHostToDevice);
@@ -2011,7 +2025,9 @@ mcx_status mcx_debug_conv3d(int32_t kind, int32_t n, int32_t dd, int32_t hh, int
     if (e == cudaSuccess) e = cudaMemcpy(bx.p, hx.data(), hx.size() * 2, cudaMemcpyHostToDevice);
     if (kind == 0) {
         hw.resize(27ull * cin * cout);
-        for (size_t i = 0; i < hw.size(); ++i) hw[i] = __float2bfloat16(w[i]);
+        for (size_t i = 0; i < hw.size(); ++i)
+            hw[packed_weight((int)(i / ((size_t)cin * cout)), (int)(i / cin % cout), (int)(i % cin), cin, cout)] =
+                __float2bfloat16(w[i]);
         if (e == cudaSuccess) e = bw.alloc(hw.size() * 2);
         if (e == cudaSuccess) e = cudaMemcpy(bw.p, hw.data(), hw.size() * 2, cudaMemcpyHostToDevice);
         if (e == cudaSuccess && bias) e = bb.alloc(cout * 4);
