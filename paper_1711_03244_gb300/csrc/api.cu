@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "mcx_internal.h"
+#include "resolve.cuh"
 
 using namespace mcxg;
 
@@ -101,39 +102,6 @@ __global__ void finalize_kernel(const double *bt, const unsigned long long *bs, 
         for (int k = 0; k < MCX_NTALLY; ++k) out_t[k] = st[0][k];
         out_t[MCX_TALLY_LAUNCHED] = n_launched;
         for (int k = 0; k < MCX_NSTAT; ++k) out_s[k] = ss[0][k];
-    }
-}
-
-// The fluence map as accumulated, in the caller's type, optionally normalised to fluence
-// rate per launched photon (x inv_norm[label], inv_norm = 1 / (mua h^3 N dt)):
-//   accum 0: the FP32 map;  accum 1 and 2: the FP64 map (accum 1 adds its block tiles
-//   into it when the walk ends).
-
-// The maps and labels carry the walk's one-voxel border ([g][nz+2][ny+2][nx+2]); the
-// output is unpadded [g][nz][ny][nx].
-template <typename T>
-__global__ void resolve_kernel(int mode, const float *hi, const double *f64,
-                               unsigned nx, unsigned ny, unsigned nvox, unsigned pnvox,
-                               unsigned n_gates, const uint8_t *labels, const float *inv_norm,
-                               T *out)
-{
-    const size_t total = (size_t)nvox * n_gates;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += stride) {
-        const unsigned v = (unsigned)(i % nvox);
-        const unsigned g = (unsigned)(i / nvox);
-        const unsigned x = v % nx, y = (v / nx) % ny, z = v / (nx * ny);
-        const unsigned pv = (unsigned)padded_index(x, y, z, nx, ny);
-        const size_t pi = (size_t)g * pnvox + pv;
-        if (mode == 0) {
-            float f = hi[pi];
-            if (inv_norm) f *= inv_norm[labels[pv]];
-            out[i] = (T)f;
-            continue;
-        }
-        double d = f64[pi];
-        if (inv_norm) d *= (double)inv_norm[labels[pv]];
-        out[i] = (T)d;
     }
 }
 
@@ -711,7 +679,6 @@ static mcx_status read_fluence_t(mcx_sim *s, T *dst, uint64_t n_elems, int32_t n
     if (!s->ran) return fail(s, MCX_E_STATE, "no run");
     DeviceGuard g(s->device);
     const uint64_t nvox = (uint64_t)s->nx * s->ny * s->nz;
-    const uint64_t pnvox = (uint64_t)(s->nx + 2) * (s->ny + 2) * (s->nz + 2);
     const uint64_t n = nvox * s->cfg.n_gates;
     if (n_elems != n) return fail(s, MCX_E_ARG, "n_elems must be n_gates*nx*ny*nz = " + std::to_string(n));
     cudaStream_t st = s->stream;
@@ -737,11 +704,16 @@ static mcx_status read_fluence_t(mcx_sim *s, T *dst, uint64_t n_elems, int32_t n
         MCX_CUDA(s, s->staging.ensure(n * sizeof(T)), "allocating the staging buffer");
         out = static_cast<T *>(s->staging.p);
     }
-    resolve_kernel<T><<<grid_for(n), 256, 0, st>>>(mode, s->fluence.as<float>(),
-                                                   s->fluence64.as<double>(), s->nx, s->ny,
-                                                   (unsigned)nvox, (unsigned)pnvox, s->cfg.n_gates,
-                                                   s->labels.as<uint8_t>(), inv_dev, out);
-    MCX_CUDA(s, cudaGetLastError(), "launching the fluence read-out");
+    // the map as accumulated: FP32 (accum 0) or FP64 (accum 2; accum 1 adds its block tiles
+    // into it when the walk ends)
+    const uint8_t *lab = s->labels.as<uint8_t>();
+    const cudaError_t re =
+        mode == kAccPlain
+            ? resolve_map<T, float, float>(s->fluence.as<float>(), s->nx, s->ny, s->nz, s->cfg.n_gates, lab,
+                                           inv_dev, out, st)
+            : resolve_map<T, double, double>(s->fluence64.as<double>(), s->nx, s->ny, s->nz, s->cfg.n_gates,
+                                             lab, inv_dev, out, st);
+    MCX_CUDA(s, re, "launching the fluence read-out");
     if (dst_on_device) return MCX_OK;
     MCX_CUDA(s, cudaMemcpyAsync(dst, out, n * sizeof(T), cudaMemcpyDeviceToHost, st),
              "copying the fluence");

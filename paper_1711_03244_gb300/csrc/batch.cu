@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "mcx_internal.h"
+#include "resolve.cuh"
 
 using namespace mcxg;
 
@@ -64,23 +65,6 @@ __global__ void batch_stats(const unsigned long long *bs, int nblocks, unsigned 
     }
     if (tid == 0)
         for (int k = 0; k < MCX_NSTAT; ++k) out[k] = ss[0][k];
-}
-
-// one simulation's map as float [g][nz][ny][nx], optionally normalised per launched
-// photon; the map and the labels carry the walk's one-voxel border
-__global__ void batch_resolve(const float *f32, const double *f64, const uint8_t *labels,
-                              const float *inv_norm, unsigned nx, unsigned ny, unsigned nvox,
-                              unsigned pnvox, size_t n, float *out)
-{
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const unsigned v = (unsigned)(i % nvox), g = (unsigned)(i / nvox);
-        const unsigned pv = (unsigned)padded_index(v % nx, (v / nx) % ny, v / (nx * ny), nx, ny);
-        const size_t pi = (size_t)g * pnvox + pv;
-        double x = f64 ? f64[pi] : (double)f32[pi];
-        if (inv_norm) x *= (double)inv_norm[labels[pv]];
-        out[i] = (float)x;
-    }
 }
 
 unsigned grid_of(size_t n)
@@ -533,11 +517,13 @@ mcx_status mcx_batch_read_fluence(mcx_batch *b, int32_t id, float *dst, uint64_t
         out = b->staging.as<float>();
     }
     const bool f64 = b->cfg.accum_mode == kAccF64;
-    batch_resolve<<<grid_of(n), 256, 0, b->stream>>>(
-        f64 ? nullptr : b->fluence.as<float>() + b->flu_off[id],
-        f64 ? b->fluence.as<double>() + b->flu_off[id] : nullptr, s->labels.as<uint8_t>(), inv,
-        s->nx, s->ny, (unsigned)nvox, (s->nx + 2) * (s->ny + 2) * (s->nz + 2), n, out);
-    BCUDA(b, cudaGetLastError(), "launching the read-out");
+    const uint8_t *lab = s->labels.as<uint8_t>();
+    const cudaError_t re =
+        f64 ? resolve_map<float, double, double>(b->fluence.as<double>() + b->flu_off[id], s->nx, s->ny, s->nz,
+                                                 b->cfg.n_gates, lab, inv, out, b->stream)
+            : resolve_map<float, float, double>(b->fluence.as<float>() + b->flu_off[id], s->nx, s->ny, s->nz,
+                                                b->cfg.n_gates, lab, inv, out, b->stream);
+    BCUDA(b, re, "launching the read-out");
     if (!dst_on_device) {
         BCUDA(b, cudaMemcpyAsync(dst, out, n * sizeof(float), cudaMemcpyDeviceToHost, b->stream), "copying");
     }
