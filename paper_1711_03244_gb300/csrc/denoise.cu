@@ -35,6 +35,7 @@
 #include <cstring>
 #include <random>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "mcx_internal.h"
@@ -250,6 +251,22 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
 }
 
+// One MMA from descriptors in two words: the low word holds the start address (in 16-byte
+// units; every address here is below 256 KiB, so sums stay in its 14 bits) and the leading
+// offset, the high word is constant per operand.  One thread issues a CTA's MMAs, and its
+// instructions between them are what spaces them: 54 clocks with one add per operand, 91
+// with 64-bit descriptors built per MMA, about 190 when the runs of accumulators were worked
+// out per MMA too; the tensor core itself needs 39 to 44 (N <= 48) and 56 (N = 96).
+__device__ __forceinline__ void mma_bf16(uint32_t d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                         uint32_t idesc, uint32_t accum)
+{
+    asm volatile("{\n .reg .b64 a, b;\n .reg .pred p;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+                 " setp.ne.b32 p, %6, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n"
+                 ::"r"(d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accum) : "memory");
+}
+__device__ __forceinline__ uint32_t lo_word(uint64_t d) { return (uint32_t)d; }
+__device__ __forceinline__ uint32_t hi_word(uint64_t d) { return (uint32_t)(d >> 32); }
+
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kTcThreads)
 conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ W,
@@ -349,10 +366,11 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
     } else if (tid == 32) {
         // ------------------------------------------------------------ MMA issuer
         if (my_units) ok &= mbar_wait(wbar, 0);
-        const uint64_t bdesc0 = umma_desc(wres, lbo_b, 128);
-        int toff[9];                                            // row offset of each (dy, dx) tap
+        const uint32_t b0 = lo_word(umma_desc(wres, lbo_b, 128)), bm0 = lo_word(umma_desc(wres, LBOM, 128));
+        const uint32_t ahi = hi_word(sw32_desc(0)), bhi = hi_word(umma_desc(0, 0, 128));
+        uint32_t toff[9];                           // each (dy, dx) tap's row offset (16-byte units)
 #pragma unroll
-        for (int tt = 0; tt < 9; ++tt) toff[tt] = (tt / 3 - 1) * PW + (tt % 3 - 1);
+        for (int tt = 0; tt < 9; ++tt) toff[tt] = (uint32_t)(2 * ((tt / 3 - 1) * PW + (tt % 3 - 1)));
         int b = 0, use = 0, T0 = 0;                             // T0: tiles of earlier units
         for (int uj = 0; uj < my_units && ok; ++uj) {
             const Unit U = unit_of(uj);
@@ -361,9 +379,7 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
                 ok &= mbar_wait(full0 + 8 * b, (uint32_t)(use & 1));
                 if (!ok) break;
                 tc_fence_after();
-                // descriptors differ only in the start-address field (address / 16, 14 bits;
-                // every address here is below 256 KiB): base descriptor plus an offset
-                const uint32_t abase = ring + (uint32_t)(b * stage_bytes + off * 32);
+                const uint32_t a0 = lo_word(sw32_desc(ring + (uint32_t)(b * stage_bytes + off * 32)));
                 if constexpr (MERGE) {
                     // tiles ilo .. ihi read this plane (tile i with dz = j - 1 - i, weight block
                     // dzi = i - j + 2); tile j starts here, tile j - 2 finishes here
@@ -374,32 +390,45 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
                         tc_fence_after();
                     }
                     if (!ok) break;
-                    const uint64_t bdm = umma_desc(wres, LBOM, 128);
-                    // one MMA for tiles a .. e (consecutive accumulators, no wrap of the ring)
-                    auto mma_run = [&](uint64_t ad, uint64_t bk, int a, int e, uint32_t accum) {
-                        const uint32_t d = tmem + (uint32_t)(((T0 + a) & (NSLOT - 1)) * NCOL);
-                        const uint64_t bd = bk + (uint64_t)(((a - j + 2) * COUT * 16) >> 4);
-                        const uint32_t idesc = idesc_bf16_f32(kTcRows, (e - a + 1) * COUT);
-                        asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                     " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                                     ::"r"(d), "l"(ad), "l"(bd), "r"(idesc), "r"(accum) : "memory");
+                    // tiles a .. e take one MMA (consecutive accumulators), two where the ring of
+                    // accumulators wraps: found once per window
+                    struct Run { uint32_t d, blo, idesc; };
+                    auto run = [&](int a, int e) {
+                        return Run{tmem + (uint32_t)(((T0 + a) & (NSLOT - 1)) * NCOL),
+                                   bm0 + (uint32_t)(((a - j + 2) * COUT * 16) >> 4),
+                                   idesc_bf16_f32(kTcRows, 0) + ((uint32_t)((e - a + 1) * COUT / 8) << 17)};
                     };
+                    auto split = [&](int a, int e) { return min(e, a + (NSLOT - 1) - ((T0 + a) & (NSLOT - 1))); };
+                    const int e1 = split(ilo, ihi);
+                    const Run r1 = run(ilo, e1), r2 = run(min(e1 + 1, ihi), ihi);
+                    auto products = [&](auto wraps) {
 #pragma unroll
-                    for (int tt = 0; tt < 9; ++tt)
+                        for (int tt = 0; tt < 9; ++tt)
 #pragma unroll
-                        for (int kk = 0; kk < CIN / 16; ++kk) {
-                            const uint64_t ad = sw32_desc(abase + (uint32_t)(toff[tt] * 32 + kk * lbo_a));
-                            const uint64_t bk = bdm + (uint64_t)((tt * 3 * wtap + 2 * kk * LBOM) >> 4);
-                            // the starting tile's first product overwrites its accumulator
-                            const bool fresh = starts && tt == 0 && kk == 0;
-                            const int last = fresh ? j - 1 : ihi;
-                            for (int a = ilo; a <= last;) {
-                                const int e = min(last, a + (NSLOT - 1) - ((T0 + a) & (NSLOT - 1)));
-                                mma_run(ad, bk, a, e, 1u);
-                                a = e + 1;
+                            for (int kk = 0; kk < CIN / 16; ++kk) {
+                                const uint32_t al = a0 + toff[tt] + (uint32_t)(kk * (lbo_a >> 4));
+                                const uint32_t bo = (uint32_t)((tt * 3 * wtap + 2 * kk * LBOM) >> 4);
+                                if (tt == 0 && kk == 0 && starts) {
+                                    // the starting tile's first product overwrites its accumulator
+                                    if (ilo < j) {
+                                        const int f1 = split(ilo, j - 1);
+                                        const Run q1 = run(ilo, f1);
+                                        mma_bf16(q1.d, al, ahi, q1.blo, bhi, q1.idesc, 1u);
+                                        if (f1 < j - 1) {
+                                            const Run q2 = run(f1 + 1, j - 1);
+                                            mma_bf16(q2.d, al, ahi, q2.blo, bhi, q2.idesc, 1u);
+                                        }
+                                    }
+                                    const Run q = run(j, j);
+                                    mma_bf16(q.d, al, ahi, q.blo, bhi, q.idesc, 0u);
+                                } else {
+                                    mma_bf16(r1.d, al, ahi, r1.blo + bo, bhi, r1.idesc, 1u);
+                                    if (decltype(wraps)::value) mma_bf16(r2.d, al, ahi, r2.blo + bo, bhi, r2.idesc, 1u);
+                                }
                             }
-                            if (fresh) mma_run(ad, bk, j, j, 0u);
-                        }
+                    };
+                    if (e1 < ihi) products(std::true_type{});
+                    else products(std::false_type{});
                     if (j >= 2) tc_commit(accf0 + 8 * ((T0 + j - 2) & (NSLOT - 1)));   // tile j - 2 is complete
                     tc_commit(empty0 + 8 * b);
                     if (++b == ns) { b = 0; ++use; }
@@ -411,19 +440,15 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
                         if (dz == -1 && T >= NSLOT)                 // the slot's previous tile is read out
                             ok &= mbar_wait(acce0 + 8 * slot, (uint32_t)((T / NSLOT - 1) & 1));
                         if (!ok) break;
-                        const uint64_t bbase = bdesc0 + (uint64_t)((9 * (dz + 1) * wtap) >> 4);
+                        const uint32_t bl = b0 + (uint32_t)((9 * (dz + 1) * wtap) >> 4);
                         const uint32_t d = tmem + slot * NCOL;
 #pragma unroll
                         for (int tt = 0; tt < 9; ++tt)              // tt = 3 (dy + 1) + (dx + 1)
 #pragma unroll
-                            for (int kk = 0; kk < CIN / 16; ++kk) {
-                                const uint64_t ad = sw32_desc(abase + (uint32_t)(toff[tt] * 32 + kk * lbo_a));
-                                const uint64_t bd = bbase + (uint64_t)((tt * wtap + 2 * kk * lbo_b) >> 4);
-                                const uint32_t accum = (dz == -1 && tt == 0 && kk == 0) ? 0u : 1u;
-                                asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                                             ::"r"(d), "l"(ad), "l"(bd), "r"(IDESC), "r"(accum) : "memory");
-                            }
+                            for (int kk = 0; kk < CIN / 16; ++kk)
+                                mma_bf16(d, a0 + toff[tt] + (uint32_t)(kk * (lbo_a >> 4)), ahi,
+                                         bl + (uint32_t)((tt * wtap + 2 * kk * lbo_b) >> 4), bhi, IDESC,
+                                         (dz == -1 && tt == 0 && kk == 0) ? 0u : 1u);
                         if (dz == 1) tc_commit(accf0 + 8 * slot);    // tile i is complete
                     }
                     tc_commit(empty0 + 8 * b);
@@ -495,9 +520,9 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
 // plane's MMAs have completed), then each tile's window of that plane streams through
 // the ring.  Weights then cross L2 once per unit and plane instead of once per tile and
 // plane.  A small volume's units hold fewer tiles (tu), so that they reach every SM.
-// Tiles, windows, operand layouts and the bounded waits are those of conv3d_fwd_tc; a
-// seventh warp loads the weights.
-constexpr int kWsHeader = 512, kWsThreads = kTcThreads + 32;    // warp 6 loads the weights
+// Tiles, windows, operand layouts and the bounded waits are those of conv3d_fwd_tc; two
+// more warps load the weights and issue every other tile's MMAs.
+constexpr int kWsHeader = 512, kWsThreads = kTcThreads + 64;    // warp 6 loads the weights, warp 7 issues MMAs
 
 __host__ __device__ constexpr int ws_tiles_per_unit(int cout)
 {
@@ -507,9 +532,11 @@ __host__ __device__ constexpr int ws_smem_bytes(int cin, int cout, int w, int ns
 {
     return 1024 + kWsHeader + 9 * cout * cin * 2 + 1024 + ns * (cin / 16) * tc_gbytes(w);
 }
+// ring depth, even: stage b always holds a window of the same MMA thread (b & 1), whose waits
+// then see each of the stage's phases in turn
 __host__ __device__ constexpr int ws_stages(int cin, int cout, int w)
 {
-    for (int ns = 6; ns >= 2; --ns)
+    for (int ns = 6; ns >= 2; ns -= 2)
         if (ws_smem_bytes(cin, cout, w, ns) <= kTcSmemMax) return ns;
     return 0;
 }
@@ -526,7 +553,7 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;      // 1 KiB aligned
     // header: full[ns] at 0, empty[ns] at 64, acc full[2 TU] at 128, acc empty[2 TU] at 256,
-    // weights full[3] at 384, weights empty[3] at 408, MMA drain at 432, TMEM address at 448
+    // weights full[3] at 384, weights empty[3] at 408, MMA drain[2] at 432, TMEM address at 448
     const uint32_t full0 = base, empty0 = base + 64, accf0 = base + 128, acce0 = base + 256;
     const uint32_t wfull = base + 384, wempty = base + 408, drain = base + 432;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem_raw + (base + 448 - smem_u32(smem_raw)));
@@ -568,9 +595,10 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
         }
         for (int r = 0; r < 3; ++r) {
             mbar_init(wfull + 8 * r, 1);
-            mbar_init(wempty + 8 * r, 1);
+            mbar_init(wempty + 8 * r, 2);
         }
         mbar_init(drain, 1);
+        mbar_init(drain + 8, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     tc_fence_before();
@@ -589,14 +617,18 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
             int t0, nt;
             unit_tiles(uj, t0, nt);
             for (int g = 0; g < 3 && ok; ++g) {               // plane z + g - 1
-                for (int t = 0; t < nt && ok; ++t) {
+                for (int t = 0; t < nt + (nt & 1) && ok; ++t) {   // an odd unit's last stage stays empty
                     if (use > 0) ok &= mbar_wait(empty0 + 8 * b, (uint32_t)((use - 1) & 1));
                     if (!ok) break;
-                    const Tl T = tile_at(t0 + t);
                     const uint32_t st = ring + b * a_bytes, fb = full0 + 8 * b;
-                    mbar_expect_tx(fb, tx);
-                    for (int c = 0; c < CIN / 16; ++c)
-                        tma_load_5d(st + c * lbo_a, &tmx, 16 * c, -1, first_line(T.q0), T.z + g - 1, T.b, fb);
+                    if (t < nt) {
+                        const Tl T = tile_at(t0 + t);
+                        mbar_expect_tx(fb, tx);
+                        for (int c = 0; c < CIN / 16; ++c)
+                            tma_load_5d(st + c * lbo_a, &tmx, 16 * c, -1, first_line(T.q0), T.z + g - 1, T.b, fb);
+                    } else {
+                        mbar_arrive(fb);
+                    }
                     if (++b == ns) { b = 0; ++use; }
                 }
             }
@@ -620,59 +652,71 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
             }
         for (int r = 0; r < 3; ++r)                           // every load has landed
             if (wloads > 0) ok &= mbar_wait(wfull + 8 * r, (uint32_t)((wloads - 1) & 1));
-    } else if (tid == 32) {
-        // ------------------------------------------------------------ MMA issuer
-        const uint64_t bdesc0 = umma_desc(wbuf, lbo_b, 128);
-        int toff[9];
+    } else if (tid == 32 || tid == kTcThreads + 32) {
+        // ------------------------------------------------------------ MMA issuers
+        // two threads, on the unit's even and odd tiles: the CTA is alone on its SM, and one
+        // thread's MMAs are 54 clocks apart at best (see mma_bf16)
+        const int me = tid == 32 ? 0 : 1;
+        const uint32_t b0 = lo_word(umma_desc(wbuf, lbo_b, 128));
+        const uint32_t ahi = hi_word(sw32_desc(0)), bhi = hi_word(umma_desc(0, 0, 128));
+        uint32_t toff[9];
 #pragma unroll
-        for (int tt = 0; tt < 9; ++tt) toff[tt] = (tt / 3 - 1) * PW + (tt % 3 - 1);
+        for (int tt = 0; tt < 9; ++tt) toff[tt] = (uint32_t)(2 * ((tt / 3 - 1) * PW + (tt % 3 - 1)));
         int b = 0, use = 0, wpass = 0;
         for (int uj = 0; uj < my_units && ok; ++uj) {
             int t0, nt;
             unit_tiles(uj, t0, nt);
             const int set = uj & 1;
             for (int g = 0; g < 3 && ok; ++g) {
-                for (int t = 0; t < nt && ok; ++t) {
-                    const int slot = set * TU + t;
-                    if (g == 0 && uj >= 2)                      // the slot's previous tile is read out
-                        ok &= mbar_wait(acce0 + 8 * slot, (uint32_t)(((uj >> 1) - 1) & 1));
-                    ok &= mbar_wait(full0 + 8 * b, (uint32_t)(use & 1));
-                    if (!ok) break;
-                    tc_fence_after();
-                    const Tl T = tile_at(t0 + t);
-                    const int off = T.q0 - first_line(T.q0) * PW;
-                    const uint32_t abase = ring + (uint32_t)(b * a_bytes + off * 32);
-                    const uint32_t d = tmem + slot * NCOL;
+                const int last = nt - 1 - ((nt - 1 - me) & 1);      // this thread's last tile (or -1)
+                for (int t = 0; t < nt + (nt & 1) && ok; ++t) {
+                    if (t == nt && (t & 1) == me) {                 // the empty stage of an odd unit
+                        ok &= mbar_wait(full0 + 8 * b, (uint32_t)(use & 1));
+                        if (ok) mbar_arrive(empty0 + 8 * b);
+                    } else if ((t & 1) == me) {
+                        const int slot = set * TU + t;
+                        if (g == 0 && uj >= 2)                      // the slot's previous tile is read out
+                            ok &= mbar_wait(acce0 + 8 * slot, (uint32_t)(((uj >> 1) - 1) & 1));
+                        ok &= mbar_wait(full0 + 8 * b, (uint32_t)(use & 1));
+                        if (!ok) break;
+                        tc_fence_after();
+                        const Tl T = tile_at(t0 + t);
+                        const int off = T.q0 - first_line(T.q0) * PW;
+                        const uint32_t a0 = lo_word(sw32_desc(ring + (uint32_t)(b * a_bytes + off * 32)));
+                        const uint32_t d = tmem + slot * NCOL;
 #pragma unroll
-                    for (int tt = 0; tt < 9; ++tt) {
-                        if (tt % 3 == 0 && t == 0) {             // this plane's weights of the group
-                            ok &= mbar_wait(wfull + 8 * (tt / 3), (uint32_t)(wpass & 1));
-                            tc_fence_after();
+                        for (int tt = 0; tt < 9; ++tt) {
+                            if (tt % 3 == 0 && t == me) {            // this plane's weights of the group
+                                ok &= mbar_wait(wfull + 8 * (tt / 3), (uint32_t)(wpass & 1));
+                                tc_fence_after();
+                                if (!ok) break;
+                            }
+#pragma unroll
+                            for (int kk = 0; kk < CIN / 16; ++kk)
+                                mma_bf16(d, a0 + toff[tt] + (uint32_t)(kk * (lbo_a >> 4)), ahi,
+                                         b0 + (uint32_t)((tt * wtap + 2 * kk * lbo_b) >> 4), bhi, IDESC,
+                                         (g == 0 && tt == 0 && kk == 0) ? 0u : 1u);
+                            if (tt % 3 == 2 && t == last) tc_commit(wempty + 8 * (tt / 3));
                         }
                         if (!ok) break;
-#pragma unroll
-                        for (int kk = 0; kk < CIN / 16; ++kk) {
-                            const uint64_t ad = sw32_desc(abase + (uint32_t)(toff[tt] * 32 + kk * lbo_a));
-                            const uint64_t bd = bdesc0 + (uint64_t)((tt * wtap + 2 * kk * lbo_b) >> 4);
-                            const uint32_t accum = (g == 0 && tt == 0 && kk == 0) ? 0u : 1u;
-                            asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                                         ::"r"(d), "l"(ad), "l"(bd), "r"(IDESC), "r"(accum) : "memory");
-                        }
-                        if (tt % 3 == 2 && t == nt - 1) tc_commit(wempty + 8 * (tt / 3));
+                        tc_commit(empty0 + 8 * b);
+                        if (g == 2) tc_commit(accf0 + 8 * slot);    // tile t of the unit is complete
                     }
-                    if (!ok) break;
-                    tc_commit(empty0 + 8 * b);
-                    if (g == 2) tc_commit(accf0 + 8 * slot);    // tile t of the unit is complete
                     if (++b == ns) { b = 0; ++use; }
+                }
+                // no tile of this plane: done with its weights, once they are there (an arrival
+                // before that would count for an earlier plane)
+                for (int r = 0; r < 3 && ok && last < 0; ++r) {
+                    ok &= mbar_wait(wfull + 8 * r, (uint32_t)(wpass & 1));
+                    if (ok) mbar_arrive(wempty + 8 * r);
                 }
                 ++wpass;
             }
         }
         // every MMA issued has completed before the CTA may free tensor memory, also when
         // a wait above gave up (the epilogue then no longer waits for the accumulators)
-        tc_commit(drain);
-        ok &= mbar_wait(drain, 0);
+        tc_commit(drain + 8 * me);
+        ok &= mbar_wait(drain + 8 * me, 0);
     } else if (warp >= 2 && warp < 6) {
         // ------------------------------------------------------------ epilogue
         const int quarter = warp & 3, r = quarter * 32 + (tid & 31);
