@@ -908,16 +908,11 @@ conv3d_wgrad_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
     } else if (warp == 1) {
         if (lane == 0) {
             // -------------------------------------------------------- MMA issuer
-            int started = 0;                                    // bit dz + 1: accumulator written
-            auto mma = [&](int dzi, uint64_t ad, uint64_t bd) {
-                const uint32_t accum = (uint32_t)((started >> dzi) & 1);
-                asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                             ::"r"(tmem + (uint32_t)(dzi * kWtN)), "l"(ad), "l"(bd), "r"(IDESC), "r"(accum)
-                             : "memory");
-                started |= 1 << dzi;
-            };
-            const uint32_t xlbo = 32, ylbo = (uint32_t)(PW * 32), sbo = 256;
+            // descriptors as in mma_bf16: both operands share the high word, the leading
+            // offsets (X 32 B, dY PW rows) sit in the low words
+            const uint32_t hi = hi_word(sw32_mn_desc(0, 32, 256));
+            const uint32_t xlo = lo_word(sw32_mn_desc(0, 32, 256)), ylo = lo_word(sw32_mn_desc(0, (uint32_t)(PW * 32), 256));
+            uint32_t on0 = 0, on1 = 0, on2 = 0;                 // accumulator of dz = -1, 0, +1 written
             int b = 0, use = 0, bp = 0;
             for (int uj = 0; uj < my_units && ok; ++uj) {
                 const Unit U = unit_of(uj);
@@ -930,18 +925,25 @@ conv3d_wgrad_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
                     tc_fence_after();
                     const bool hasy = j >= 1 && j <= U.nz, prevy = j >= 2;
                     const uint32_t xs = ring + b * stage_bytes, xp = ring + bp * stage_bytes;
-                    const uint32_t ys = xs + xbytes, yp = xp + xbytes;
-#pragma unroll 1
-                    for (int kk = 0; kk < kTcRows / 16; ++kk) {
-                        const uint32_t ko = (uint32_t)(kk * 16 * 32);
-                        const uint64_t ax = sw32_mn_desc(xs + rx + ko, xlbo, sbo);
-                        if (hasy) {
-                            const uint64_t ay = sw32_mn_desc(ys + ry + ko, ylbo, sbo);
-                            mma(1, ax, ay);                                          // dz = 0
-                            mma(0, sw32_mn_desc(xp + rx + ko, xlbo, sbo), ay);         // dz = -1
+                    const uint32_t ax = xlo + ((xs + rx) >> 4), axp = xlo + ((xp + rx) >> 4);
+                    const uint32_t ay = ylo + ((xs + xbytes + ry) >> 4), ayp = ylo + ((xp + xbytes + ry) >> 4);
+                    auto products = [&](auto has, auto prev) {
+#pragma unroll
+                        for (int kk = 0; kk < kTcRows / 16; ++kk) {
+                            const uint32_t ko = (uint32_t)(kk * 32);       // 16 rows of 32 B
+                            if (decltype(has)::value) {
+                                mma_bf16(tmem + kWtN, ax + ko, hi, ay + ko, hi, IDESC, kk ? 1u : on1);   // dz = 0
+                                mma_bf16(tmem, axp + ko, hi, ay + ko, hi, IDESC, kk ? 1u : on0);         // dz = -1
+                            }
+                            if (decltype(prev)::value)
+                                mma_bf16(tmem + 2 * kWtN, ax + ko, hi, ayp + ko, hi, IDESC, kk ? 1u : on2);   // +1
                         }
-                        if (prevy) mma(2, ax, sw32_mn_desc(yp + ry + ko, ylbo, sbo));  // dz = +1
-                    }
+                    };
+                    if (hasy && prevy) products(std::true_type{}, std::true_type{});
+                    else if (hasy) products(std::true_type{}, std::false_type{});
+                    else if (prevy) products(std::false_type{}, std::true_type{});
+                    if (hasy) on0 = on1 = 1;
+                    if (prevy) on2 = 1;
                     if (j >= 1) tc_commit(empty0 + 8 * bp);             // the previous plane is done
                     if (j == U.nz + 1) tc_commit(empty0 + 8 * b);       // and so is the unit's last
                     bp = b;
