@@ -1045,13 +1045,28 @@ __device__ __forceinline__ void children_of(int pc, const Vol &vf, int *ch)
 #define GRID_LOOP(i, n) \
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += gridDim.x * blockDim.x)
 
-// ReLU backward fused with the bias gradient: zero dY where the stored output is not
-// positive and add what survives into db[channel].  Chunk i holds channels
+// ReLU backward fused with the bias gradient and with what produces the gradient, so that it
+// is written once: zero dY where the stored output is not positive and add what survives
+// into db[channel].  The gradient of position p comes from
+//   kGradPlain     dY itself (an input-gradient convolution wrote it);
+//   kGradPoolSkip  the pooled gradient's parent / 8 plus the skip channels of gcat
+//                  (cx + C channels per fine position);
+//   kGradUp        the sum of the 8 children's first C channels of gcat (cx + cs channels
+//                  per fine position, C = cx).
+// Each intermediate is rounded to BF16 as when it was stored.  Chunk i holds channels
 // 8 (i mod C/8) .. +7 of position i / (C/8); the grid stride is a multiple of 256 chunks,
 // so each thread keeps one 8-channel group and sums it in registers, then lanes of the
-// same group, then the block's warps, with one atomic per channel per block.
-template <int C>
-__global__ void __launch_bounds__(256) relu_bias_grad(bf16 *dY, const bf16 *Y, int n8, float *db)
+// same group, then the block's warps, with one atomic per channel per block.  Memory-bound
+// (4 volumes of 64^3, 16 channels: pool, skip and ReLU as three passes took 50 us).
+enum { kGradPlain = 0, kGradPoolSkip = 1, kGradUp = 2 };
+struct GradSource {
+    const bf16 *pooled, *gcat;
+    int ccat, cx;                 // channels of gcat, and those before the skip
+    Vol v;                        // this layer's volume
+};
+
+template <int C, int SRC>
+__global__ void __launch_bounds__(256) relu_bias_grad(bf16 *dY, const bf16 *Y, int n8, float *db, const GradSource S)
 {
     static_assert(C % 8 == 0 && 32 % (C / 8) == 0, "8-channel groups must tile a warp");
     constexpr int G = C / 8;
@@ -1060,7 +1075,33 @@ __global__ void __launch_bounds__(256) relu_bias_grad(bf16 *dY, const bf16 *Y, i
     GRID_LOOP(i, n8) {
         float y[8], g[8];
         Bf8{ld16(Y + 8 * (size_t)i)}.to(y);
-        Bf8{ld16(dY + 8 * (size_t)i)}.to(g);
+        const int p = i / G, j = i - p * G;
+        if (SRC == kGradPlain) {
+            Bf8{ld16(dY + 8 * (size_t)i)}.to(g);
+        } else if (SRC == kGradPoolSkip) {
+            float k[8];
+            Bf8{ld16(S.pooled + (size_t)parent_of(p, S.v) * C + 8 * j)}.to(g);
+            Bf8{ld16(S.gcat + (size_t)p * S.ccat + S.cx + 8 * j)}.to(k);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) g[e] *= 0.125f;
+            Bf8::from(g).to(g);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) g[e] += k[e];
+            Bf8::from(g).to(g);
+        } else {
+            int ch[8];
+            children_of(p, Vol{S.v.n, 2 * S.v.d, 2 * S.v.h, 2 * S.v.w}, ch);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) g[e] = 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                float f[8];
+                Bf8{ld16(S.gcat + (size_t)ch[k] * S.ccat + 8 * j)}.to(f);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) g[e] += f[e];
+            }
+            Bf8::from(g).to(g);
+        }
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             if (y[k] <= 0.f) g[k] = 0.f;
@@ -1204,20 +1245,6 @@ __global__ void avgpool_fwd(const bf16 *X, Vol vo, int c, bf16 *Y)
     }
 }
 
-// gradient of the pooling: each fine position gets its parent's gradient / 8
-__global__ void avgpool_bwd(const bf16 *dY, Vol vi, int c, bf16 *dX)
-{
-    const int c8 = c / 8, n = vi.n * vi.d * vi.h * vi.w * c8;
-    GRID_LOOP(i, n) {
-        const int p = i / c8, j = i - p * c8;
-        float f[8];
-        Bf8{ld16(dY + (size_t)parent_of(p, vi) * c + 8 * j)}.to(f);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) f[e] *= 0.125f;
-        st16(dX + (size_t)p * c + 8 * j, Bf8::from(f).u);
-    }
-}
-
 // nearest x2 upsampling of X (coarse, cx channels) into channels [0, cx) of the fine
 // volume vf, and the skip S (cs channels) into channels [cx, cx + cs)
 __global__ void upcat_fwd(const bf16 *X, int cx, const bf16 *S, int cs, Vol vf, bf16 *Y)
@@ -1228,42 +1255,6 @@ __global__ void upcat_fwd(const bf16 *X, int cx, const bf16 *S, int cs, Vol vf, 
         const uint4 v = j < x8 ? ld16(X + (size_t)parent_of(p, vf) * cx + 8 * j)
                                : ld16(S + (size_t)p * cs + 8 * (j - x8));
         st16(Y + (size_t)p * (cx + cs) + 8 * j, v);
-    }
-}
-
-// gradient of upcat, coarse part: each coarse position sums its 8 children
-__global__ void upcat_bwd_coarse(const bf16 *dY, int cx, int cs, Vol vc, bf16 *dX)
-{
-    const int c = cx + cs, x8 = cx / 8, n = vc.n * vc.d * vc.h * vc.w * x8;
-    const Vol vf{vc.n, 2 * vc.d, 2 * vc.h, 2 * vc.w};
-    GRID_LOOP(i, n) {
-        const int pc = i / x8, j = i - pc * x8;
-        int ch[8];
-        children_of(pc, vf, ch);
-        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            float f[8];
-            Bf8{ld16(dY + (size_t)ch[k] * c + 8 * j)}.to(f);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] += f[e];
-        }
-        st16(dX + (size_t)pc * cx + 8 * j, Bf8::from(acc).u);
-    }
-}
-
-// gradient of upcat, skip part, added to dS
-__global__ void upcat_bwd_skip_add(const bf16 *dY, int cx, int cs, int npos, bf16 *dS)
-{
-    const int c = cx + cs, s8 = cs / 8, n = npos * s8;
-    GRID_LOOP(i, n) {
-        const int p = i / s8, j = i - p * s8;
-        float a[8], b[8];
-        Bf8{ld16(dS + (size_t)p * cs + 8 * j)}.to(a);
-        Bf8{ld16(dY + (size_t)p * c + cx + 8 * j)}.to(b);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) a[e] += b[e];
-        st16(dS + (size_t)p * cs + 8 * j, Bf8::from(a).u);
     }
 }
 
@@ -1281,11 +1272,12 @@ __global__ void head_fwd(const bf16 *Y, const float *x, const float *hw, const f
     }
 }
 
-// loss L = mean (out - target)^2, dout = 2 (out - target) / n; dY = dout hw; head grads
+// loss L = mean (out - target)^2, dout = 2 (out - target) / n; dY = dout hw where the last
+// layer's output Y is positive (its ReLU), and that layer's bias gradient db; head grads
 __global__ void head_bwd(const bf16 *Y, const float *out, const float *target, const float *hw, int npos,
-                         bf16 *dY, float *dhw, float *dhb, float *loss)
+                         bf16 *dY, float *dhw, float *dhb, float *loss, float *db)
 {
-    float gw[16] = {0}, gb = 0.f, l = 0.f;
+    float gw[16] = {0}, gd[16] = {0}, gb = 0.f, l = 0.f;
     const float inv_n = 1.f / (float)npos;
     GRID_LOOP(p, npos) {
         const float e = out[p] - target[p];
@@ -1300,28 +1292,43 @@ __global__ void head_bwd(const bf16 *Y, const float *out, const float *target, c
             gw[c] += d * y[c];
             g[c] = d * hw[c];
         }
+        Bf8 lo = Bf8::from(g), hi = Bf8::from(g + 8);
+        lo.to(g);
+        hi.to(g + 8);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+            if (y[c] <= 0.f) g[c] = 0.f;
+            gd[c] += g[c];
+        }
         st16(dY + 16 * (size_t)p, Bf8::from(g).u);
         st16(dY + 16 * (size_t)p + 8, Bf8::from(g + 8).u);
     }
-    // warp sums, then block sums in shared memory: 18 atomics per block
-    __shared__ float red[8][18];
+    // warp sums, then block sums in shared memory: 34 atomics per block
+    __shared__ float red[8][34];
     for (int o = 16; o > 0; o >>= 1) {
         l += __shfl_down_sync(0xffffffffu, l, o);
         gb += __shfl_down_sync(0xffffffffu, gb, o);
 #pragma unroll
-        for (int c = 0; c < 16; ++c) gw[c] += __shfl_down_sync(0xffffffffu, gw[c], o);
+        for (int c = 0; c < 16; ++c) {
+            gw[c] += __shfl_down_sync(0xffffffffu, gw[c], o);
+            gd[c] += __shfl_down_sync(0xffffffffu, gd[c], o);
+        }
     }
     const int w = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) {
         red[w][0] = l;
         red[w][1] = gb;
-        for (int c = 0; c < 16; ++c) red[w][2 + c] = gw[c];
+        for (int c = 0; c < 16; ++c) {
+            red[w][2 + c] = gw[c];
+            red[w][18 + c] = gd[c];
+        }
     }
     __syncthreads();
-    if (threadIdx.x < 18) {
+    if (threadIdx.x < 34) {
         float t = 0.f;
         for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k][threadIdx.x];
-        atomicAdd(threadIdx.x == 0 ? loss : threadIdx.x == 1 ? dhb : dhw + (threadIdx.x - 2), t);
+        atomicAdd(threadIdx.x == 0 ? loss : threadIdx.x == 1 ? dhb
+                  : threadIdx.x < 18 ? dhw + (threadIdx.x - 2) : db + (threadIdx.x - 18), t);
     }
 }
 
@@ -1340,18 +1347,23 @@ __global__ void adam_step(float *w, const float *gr, float *m, float *v, long lo
     }
 }
 
-// the BF16 copies of a convolution's weights, packed: [tap][co][ci] for the forward pass and
-// [26 - tap][ci][co] for the input gradient
-__global__ void refresh_conv_bf16(const float *w, int cin, int cout, bf16 *wf, bf16 *wb)
+// the BF16 copies of the convolutions' weights, packed: [tap][co][ci] for the forward pass
+// and [26 - tap][ci][co] for the input gradient; blockIdx.y = layer (ten launches of a few
+// microseconds each took 37 us of a training step)
+struct RefreshList {
+    const float *w[10];
+    bf16 *wf[10], *wb[10];
+    int cin[10], cout[10];
+};
+
+__global__ void refresh_conv_bf16(const RefreshList L)
 {
-    const long long n = 27LL * cin * cout, st = (long long)gridDim.x * blockDim.x;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += st) {
-        const int ci = (int)(i % cin);
-        const int co = (int)((i / cin) % cout);
-        const int tap = (int)(i / ((long long)cin * cout));
-        const bf16 b = __float2bfloat16(w[i]);
-        wf[packed_weight(tap, co, ci, cin, cout)] = b;
-        wb[packed_weight(26 - tap, ci, co, cout, cin)] = b;
+    const int l = blockIdx.y, cin = L.cin[l], cout = L.cout[l], n = 27 * cin * cout;
+    GRID_LOOP(i, n) {
+        const int ci = i % cin, co = i / cin % cout, tap = i / (cin * cout);
+        const bf16 b = __float2bfloat16(L.w[l][i]);
+        L.wf[l][packed_weight(tap, co, ci, cin, cout)] = b;
+        L.wb[l][packed_weight(26 - tap, ci, co, cout, cin)] = b;
     }
 }
 
@@ -1658,11 +1670,15 @@ static Vol level_vol(const mcx_denoiser *d, int level, int n)
 
 static mcx_status refresh_weights(mcx_denoiser *d, cudaStream_t st)
 {
+    RefreshList R;
     for (int l = 0; l < 10; ++l) {
-        const LayerSpec &L = kLayers[l];
-        refresh_conv_bf16<<<grid1(27LL * L.cin * L.cout), 256, 0, st>>>(
-            d->params.as<float>() + d->w_off[l], L.cin, L.cout, d->wf[l].as<bf16>(), d->wb[l].as<bf16>());
+        R.w[l] = d->params.as<float>() + d->w_off[l];
+        R.wf[l] = d->wf[l].as<bf16>();
+        R.wb[l] = d->wb[l].as<bf16>();
+        R.cin[l] = kLayers[l].cin;
+        R.cout[l] = kLayers[l].cout;
     }
+    refresh_conv_bf16<<<dim3(64, 10), 256, 0, st>>>(R);
     DNC(d, cudaGetLastError(), "refreshing BF16 weights");
     return MCX_OK;
 }
@@ -1707,23 +1723,31 @@ static mcx_status forward(mcx_denoiser *d, const float *x, const float *aux, int
     return MCX_OK;
 }
 
-// backward of a conv layer l with input `in`: dA (gradient of its ReLU output, in place in
-// ga[l]) -> weight and bias gradients, and (if dIn) the input gradient
+// ReLU backward and bias gradient of layer l: from its output's gradient in ga[l], or from
+// the gradients that src forms it of
+static mcx_status relu_bwd(mcx_denoiser *d, int l, Vol v, int src, GradSource S, cudaStream_t st)
+{
+    const int C = kLayers[l].cout, n8 = (int)(v.pos() * C / 8);
+    const unsigned rb = std::min(grid1(n8), 152u * 4u);
+    bf16 *dA = d->ga[l].as<bf16>();
+    const bf16 *A = d->a[l].as<bf16>();
+    float *db = d->grads.as<float>() + d->b_off[l];
+    S.v = v;
+#define MCX_RB(c, k) \
+    if (C == c && src == k) { relu_bias_grad<c, k><<<rb, 256, 0, st>>>(dA, A, n8, db, S); return MCX_OK; }
+    MCX_RB(16, kGradPlain) MCX_RB(32, kGradPlain) MCX_RB(64, kGradPlain)
+    MCX_RB(16, kGradPoolSkip) MCX_RB(32, kGradPoolSkip) MCX_RB(32, kGradUp) MCX_RB(64, kGradUp)
+#undef MCX_RB
+    return dn_fail(d, MCX_E_STATE, "no ReLU/bias-gradient kernel for this channel count");
+}
+
+// backward of a conv layer l with input `in`: dA (gradient of its output before the ReLU, in
+// ga[l]) -> weight gradient, and (if dIn) the input gradient
 static mcx_status conv_bwd(mcx_denoiser *d, int l, const bf16 *in, Vol v, bf16 *dIn, cudaStream_t st)
 {
     const LayerSpec &L = kLayers[l];
     float *G = d->grads.as<float>();
     bf16 *dA = d->ga[l].as<bf16>();
-    const int n8 = (int)(v.pos() * L.cout / 8);
-    const unsigned rb = std::min(grid1(n8), 152u * 4u);
-    const bf16 *A = d->a[l].as<bf16>();
-    float *db = G + d->b_off[l];
-    switch (L.cout) {
-    case 16: relu_bias_grad<16><<<rb, 256, 0, st>>>(dA, A, n8, db); break;
-    case 32: relu_bias_grad<32><<<rb, 256, 0, st>>>(dA, A, n8, db); break;
-    case 64: relu_bias_grad<64><<<rb, 256, 0, st>>>(dA, A, n8, db); break;
-    default: return dn_fail(d, MCX_E_STATE, "no ReLU/bias-gradient kernel for this channel count");
-    }
     DNC(d, launch_bwd_w(in, L.cin, dA, L.cout, v, G + d->w_off[l], d->status.as<unsigned>(), st), "weight gradient");
     if (dIn)
         DNC(d, launch_fwd_tc(dA, L.cout, d->wb[l].as<bf16>(), nullptr, v, L.cin, 0, dIn, d->status.as<unsigned>(), st),
@@ -1740,25 +1764,33 @@ static mcx_status backward(mcx_denoiser *d, const float *x, const float *target,
     DNC(d, cudaMemsetAsync(d->loss.p, 0, sizeof(float), st), "clearing the loss");
     head_bwd<<<std::min(grid1(v0.pos()), 152u * 8u), 256, 0, st>>>(d->a[9].as<bf16>(), d->out.as<float>(), target,
                                              P + d->hw_off, (int)v0.pos(), d->ga[9].as<bf16>(),
-                                             G + d->hw_off, G + d->hb_off, d->loss.as<float>());
+                                             G + d->hw_off, G + d->hb_off, d->loss.as<float>(), G + d->b_off[9]);
     mcx_status s;
+    const bf16 *gu1 = d->gu1.as<bf16>(), *gu2 = d->gu2.as<bf16>();
+    const GradSource none{}, up1{nullptr, gu1, 48, 0, {}}, up2{nullptr, gu2, 96, 0, {}};
+    const GradSource pool1{d->gp1.as<bf16>(), gu1, 48, 32, {}}, pool2{d->gp2.as<bf16>(), gu2, 96, 64, {}};
+#define MCX_RELU(l, v, src, S) if ((s = relu_bwd(d, l, v, src, S, st)) != MCX_OK) return s
     if ((s = conv_bwd(d, 9, d->a[8].as<bf16>(), v0, d->ga[8].as<bf16>(), st)) != MCX_OK) return s;
+    MCX_RELU(8, v0, kGradPlain, none);
     if ((s = conv_bwd(d, 8, d->u1.as<bf16>(), v0, d->gu1.as<bf16>(), st)) != MCX_OK) return s;
-    // upcat 1: coarse part -> d2b output gradient, skip part -> e1b output gradient (later)
-    upcat_bwd_coarse<<<grid1(v1.pos() * 4), 256, 0, st>>>(d->gu1.as<bf16>(), 32, 16, v1, d->ga[7].as<bf16>());
+    // upcat 1: coarse part -> d2b's output, skip part -> e1b's output (later)
+    MCX_RELU(7, v1, kGradUp, up1);
     if ((s = conv_bwd(d, 7, d->a[6].as<bf16>(), v1, d->ga[6].as<bf16>(), st)) != MCX_OK) return s;
+    MCX_RELU(6, v1, kGradPlain, none);
     if ((s = conv_bwd(d, 6, d->u2.as<bf16>(), v1, d->gu2.as<bf16>(), st)) != MCX_OK) return s;
-    upcat_bwd_coarse<<<grid1(v2.pos() * 8), 256, 0, st>>>(d->gu2.as<bf16>(), 64, 32, v2, d->ga[5].as<bf16>());
+    MCX_RELU(5, v2, kGradUp, up2);
     if ((s = conv_bwd(d, 5, d->a[4].as<bf16>(), v2, d->ga[4].as<bf16>(), st)) != MCX_OK) return s;
+    MCX_RELU(4, v2, kGradPlain, none);
     if ((s = conv_bwd(d, 4, d->p2.as<bf16>(), v2, d->gp2.as<bf16>(), st)) != MCX_OK) return s;
-    // e2b output gradient = pool backward + the skip part of upcat 2
-    avgpool_bwd<<<grid1(v1.pos() * 4), 256, 0, st>>>(d->gp2.as<bf16>(), v1, 32, d->ga[3].as<bf16>());
-    upcat_bwd_skip_add<<<grid1(v1.pos() * 4), 256, 0, st>>>(d->gu2.as<bf16>(), 64, 32, (int)v1.pos(), d->ga[3].as<bf16>());
+    // e2b's output: the pool's gradient + the skip part of upcat 2
+    MCX_RELU(3, v1, kGradPoolSkip, pool2);
     if ((s = conv_bwd(d, 3, d->a[2].as<bf16>(), v1, d->ga[2].as<bf16>(), st)) != MCX_OK) return s;
+    MCX_RELU(2, v1, kGradPlain, none);
     if ((s = conv_bwd(d, 2, d->p1.as<bf16>(), v1, d->gp1.as<bf16>(), st)) != MCX_OK) return s;
-    avgpool_bwd<<<grid1(v0.pos() * 2), 256, 0, st>>>(d->gp1.as<bf16>(), v0, 16, d->ga[1].as<bf16>());
-    upcat_bwd_skip_add<<<grid1(v0.pos() * 2), 256, 0, st>>>(d->gu1.as<bf16>(), 32, 16, (int)v0.pos(), d->ga[1].as<bf16>());
+    MCX_RELU(1, v0, kGradPoolSkip, pool1);
     if ((s = conv_bwd(d, 1, d->a[0].as<bf16>(), v0, d->ga[0].as<bf16>(), st)) != MCX_OK) return s;
+    MCX_RELU(0, v0, kGradPlain, none);
+#undef MCX_RELU
     if (d->n_aux == 0)                  // the forward pass used the direct input layer
         pad_input<<<grid1(v0.pos()), 256, 0, st>>>(x, nullptr, 0, d->D * d->H * d->W, (int)v0.pos(),
                                                   d->x16.as<bf16>());
