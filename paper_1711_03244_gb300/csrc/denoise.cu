@@ -1145,27 +1145,31 @@ __global__ void pad_input(const float *x, const float *aux, int n_aux, int vol, 
 // outputs of 4 consecutive positions of a line (the width is a multiple of 16) from the
 // FP32 input, rounded to BF16 as the padded path stores it, with FP32 sums on the CUDA
 // cores: each input line segment is loaded once per (dz, dy) and each 4-channel weight
-// vector (shared memory) serves 16 products
+// vector (shared memory) serves 16 products.  Two channels per packed FMA: the kernel is
+// bound by issue, and these are most of its instructions
 constexpr int kInThreads = 256;
 __global__ void __launch_bounds__(kInThreads, 2)
 conv_in_fwd(const float *__restrict__ x, const bf16 *__restrict__ W, const float *__restrict__ bias, Vol v,
             bf16 *__restrict__ Y)
 {
-    __shared__ float4 sw[27][4];                  // W[tap][co][ci = 0], 4 channels per float4
+    __shared__ __align__(16) float sw[27][16];    // W[tap][co][ci = 0]
     __shared__ float sb[16];
     for (int i = threadIdx.x; i < 27 * 16; i += blockDim.x)
-        reinterpret_cast<float *>(sw)[i] = __bfloat162float(W[packed_weight(i / 16, i % 16, 0, 16, 16)]);
+        sw[i / 16][i % 16] = __bfloat162float(W[packed_weight(i / 16, i % 16, 0, 16, 16)]);
     if (threadIdx.x < 16) sb[threadIdx.x] = bias ? bias[threadIdx.x] : 0.f;
     __syncthreads();
     const int nquad = (int)(v.pos() / 4), wq = v.w / 4;
     auto rnd = [](float f) { return __bfloat162float(__float2bfloat16(f)); };
+    auto pack = [](float lo, float hi) {
+        return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+    };
     GRID_LOOP(qd, nquad) {
         const int x0 = 4 * (qd % wq), r1 = qd / wq, yy = r1 % v.h, r2 = r1 / v.h, zz = r2 % v.d, b = r2 / v.d;
-        float acc[4][16];
+        unsigned long long acc[4][8];                 // channels 2c and 2c + 1
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int co = 0; co < 16; ++co) acc[i][co] = sb[co];
+            for (int c = 0; c < 8; ++c) acc[i][c] = pack(sb[2 * c], sb[2 * c + 1]);
 #pragma unroll
         for (int dz = -1; dz <= 1; ++dz) {
             const int z2 = zz + dz;
@@ -1181,19 +1185,19 @@ conv_in_fwd(const float *__restrict__ x, const bf16 *__restrict__ W, const float
                     if (x0 > 0) xs[0] = rnd(__ldg(line + x0 - 1));
                     if (x0 + 4 < v.w) xs[5] = rnd(__ldg(line + x0 + 4));
                 }
+                unsigned long long xx[6];
+#pragma unroll
+                for (int i = 0; i < 6; ++i) xx[i] = pack(xs[i], xs[i]);
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx) {
                     const int t = 9 * (dz + 1) + 3 * (dy + 1) + dx;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float4 wv = sw[t][q];
+                    for (int c = 0; c < 8; c += 2) {
+                        const ulonglong2 wv = *reinterpret_cast<const ulonglong2 *>(&sw[t][2 * c]);
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const float xv = xs[i + dx];
-                            acc[i][4 * q] = fmaf(xv, wv.x, acc[i][4 * q]);
-                            acc[i][4 * q + 1] = fmaf(xv, wv.y, acc[i][4 * q + 1]);
-                            acc[i][4 * q + 2] = fmaf(xv, wv.z, acc[i][4 * q + 2]);
-                            acc[i][4 * q + 3] = fmaf(xv, wv.w, acc[i][4 * q + 3]);
+                            asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][c]) : "l"(xx[i + dx]), "l"(wv.x));
+                            asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][c + 1]) : "l"(xx[i + dx]), "l"(wv.y));
                         }
                     }
                 }
@@ -1202,10 +1206,14 @@ conv_in_fwd(const float *__restrict__ x, const bf16 *__restrict__ W, const float
         bf16 *yo = Y + 16 * ((size_t)qd * 4);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
+            float o[16];
 #pragma unroll
-            for (int co = 0; co < 16; ++co) acc[i][co] = fmaxf(acc[i][co], 0.f);
-            st16(yo + 16 * i, Bf8::from(acc[i]).u);
-            st16(yo + 16 * i + 8, Bf8::from(acc[i] + 8).u);
+            for (int c = 0; c < 8; ++c) {
+                o[2 * c] = fmaxf(__uint_as_float((unsigned)acc[i][c]), 0.f);
+                o[2 * c + 1] = fmaxf(__uint_as_float((unsigned)(acc[i][c] >> 32)), 0.f);
+            }
+            st16(yo + 16 * i, Bf8::from(o).u);
+            st16(yo + 16 * i + 8, Bf8::from(o + 8).u);
         }
     }
 }
