@@ -52,6 +52,29 @@ __device__ __forceinline__ unsigned pack_bf16(float lo, float hi)
     return *reinterpret_cast<const unsigned *>(&v);
 }
 
+struct Bf8 {
+    uint4 u;
+    __device__ void to(float *f) const
+    {
+        const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 t = __bfloat1622float2(h[i]);
+            f[2 * i] = t.x;
+            f[2 * i + 1] = t.y;
+        }
+    }
+    __device__ static Bf8 from(const float *f)
+    {
+        Bf8 r;
+        r.u.x = pack_bf16(f[0], f[1]);
+        r.u.y = pack_bf16(f[2], f[3]);
+        r.u.z = pack_bf16(f[4], f[5]);
+        r.u.w = pack_bf16(f[6], f[7]);
+        return r;
+    }
+};
+
 struct Vol {
     int n, d, h, w;               // batch, depth (z), height (y), width (x)
     __host__ __device__ long long pos() const { return (long long)n * d * h * w; }
@@ -251,6 +274,14 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
 }
 
+// The network's last layer forms the output in its epilogue, where a thread holds a position's
+// 16 channels: out[p] = x[p] + hb + sum_c hw[c] Y[p][c] (Y as rounded to BF16).  out = NULL:
+// no head.  Without Y (nothing reads the layer back) its store goes too.
+struct Head {
+    const float *hw, *hb, *x;
+    float *out;
+};
+
 // One MMA from descriptors in two words: the low word holds the start address (in 16-byte
 // units; every address here is below 256 KiB, so sums stay in its 14 bits) and the leading
 // offset, the high word is constant per operand.  One thread issues a CTA's MMAs, and its
@@ -269,9 +300,9 @@ __device__ __forceinline__ uint32_t hi_word(uint64_t d) { return (uint32_t)(d >>
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kTcThreads)
-conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ W,
-              const float *__restrict__ bias, Vol v, int relu, bf16 *__restrict__ Y, unsigned *err, int ns,
-              int zc)
+conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmx2, int g1,
+              const bf16 *__restrict__ W, const float *__restrict__ bias, Vol v, int relu, bf16 *__restrict__ Y,
+              unsigned *err, int ns, int zc, const Head head)
 {
     constexpr int cin = CIN;
     static_assert(tc_wall(CIN, COUT), "larger weights take conv3d_fwd_ws");
@@ -338,6 +369,7 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
     if (tid == 0) {
         // ------------------------------------------------------------ producer (TMA)
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmx2)) : "memory");
         if (my_units) {
             mbar_expect_tx(wbar, 27 * wtap);
             bulk_load(wres, W, 27 * wtap, wbar);
@@ -353,7 +385,8 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
                 const uint32_t st = ring + b * stage_bytes, fb = full0 + 8 * b;
                 mbar_expect_tx(fb, tx);
                 for (int c = 0; c < cin / 16; ++c)
-                    tma_load_5d(st + c * lbo_a, &tmx, 16 * c, -1, fl, U.z0 - 1 + j, U.b, fb);
+                    tma_load_5d(st + c * lbo_a, c < g1 ? &tmx : &tmx2, 16 * (c < g1 ? c : c - g1), -1, fl,
+                                U.z0 - 1 + j, U.b, fb);
                 if (++b == ns) { b = 0; ++use; }
             }
         }
@@ -483,7 +516,10 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
                 tc_fence_before();
                 mbar_arrive(acce0 + 8 * slot);
                 if (valid) {
-                    bf16 *yr = Y + ((((long long)U.b * v.d + U.z0 + i) * v.h + y) * v.w + x) * COUT;
+                    const long long p = (((long long)U.b * v.d + U.z0 + i) * v.h + y) * v.w + x;
+                    bf16 *yr = Y + p * COUT;
+                    float hs = 0.f;
+                    if (COUT == 16 && head.out) hs = __ldg(head.hb);
 #pragma unroll
                     for (int c = 0; c < COUT; c += 8) {
                         float o[8];
@@ -497,8 +533,14 @@ conv3d_fwd_tc(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
                         pk.y = pack_bf16(o[2], o[3]);
                         pk.z = pack_bf16(o[4], o[5]);
                         pk.w = pack_bf16(o[6], o[7]);
-                        *reinterpret_cast<uint4 *>(yr + c) = pk;
+                        if (COUT != 16 || Y) *reinterpret_cast<uint4 *>(yr + c) = pk;
+                        if (COUT == 16 && head.out) {
+                            Bf8{pk}.to(o);
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) hs = fmaf(__ldg(head.hw + c + e), o[e], hs);
+                        }
                     }
+                    if (COUT == 16 && head.out) head.out[p] = head.x[p] + hs;
                 }
             }
         }
@@ -543,8 +585,8 @@ __host__ __device__ constexpr int ws_stages(int cin, int cout, int w)
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kWsThreads)
-conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ W,
-              const float *__restrict__ bias, Vol v, int relu, bf16 *__restrict__ Y, unsigned *err, int ns,
+conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmx2, int g1,
+              const bf16 *__restrict__ W, const float *__restrict__ bias, Vol v, int relu, bf16 *__restrict__ Y, unsigned *err, int ns,
               int tu)
 {
     constexpr int NCOL = COUT <= 32 ? 32 : (COUT <= 64 ? 64 : 128);   // TMEM columns per accumulator
@@ -611,6 +653,7 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
     if (tid == 0) {
         // ------------------------------------------------------------ producer (TMA)
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmx2)) : "memory");
         const uint32_t tx = (CIN / 16) * (L * PW * 32);
         int b = 0, use = 0;
         for (int uj = 0; uj < my_units && ok; ++uj) {
@@ -625,7 +668,8 @@ conv3d_fwd_ws(const __grid_constant__ CUtensorMap tmx, const bf16 *__restrict__ 
                         const Tl T = tile_at(t0 + t);
                         mbar_expect_tx(fb, tx);
                         for (int c = 0; c < CIN / 16; ++c)
-                            tma_load_5d(st + c * lbo_a, &tmx, 16 * c, -1, first_line(T.q0), T.z + g - 1, T.b, fb);
+                            tma_load_5d(st + c * lbo_a, c < g1 ? &tmx : &tmx2, 16 * (c < g1 ? c : c - g1), -1,
+                                        first_line(T.q0), T.z + g - 1, T.b, fb);
                     } else {
                         mbar_arrive(fb);
                     }
@@ -826,8 +870,8 @@ __device__ __forceinline__ uint64_t sw32_mn_desc(uint32_t saddr, uint32_t lbo, u
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kWtThreads)
-conv3d_wgrad_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmdy, Vol v, int ns,
-                int zc, float *__restrict__ dW, unsigned *err)
+conv3d_wgrad_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmx2, int g1,
+                const __grid_constant__ CUtensorMap tmdy, Vol v, int ns, int zc, float *__restrict__ dW, unsigned *err)
 {
     constexpr int NG = COUT / 16;
     // kind::f16, M = 64, N = 48, A and B both MN-major (bits 15 and 16)
@@ -881,6 +925,7 @@ conv3d_wgrad_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
         if (lane == 0) {
             // -------------------------------------------------------- producer (TMA)
             asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmx2)) : "memory");
             asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmdy)) : "memory");
             const uint32_t txx = (uint32_t)(Lx * PW * 32), txy = (uint32_t)(Ly * PW * 32);
             int b = 0, use = 0;
@@ -893,7 +938,8 @@ conv3d_wgrad_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
                     if (!ok) break;
                     const uint32_t st = ring + b * stage_bytes, fb = full0 + 8 * b;
                     mbar_expect_tx(fb, txx + (hasy ? txy : 0u));
-                    tma_load_5d(st, &tmx, 16 * cig, -1, xl, U.z0 - 1 + j, U.b, fb);
+                    tma_load_5d(st, cig < g1 ? &tmx : &tmx2, 16 * (cig < g1 ? cig : cig - g1), -1, xl, U.z0 - 1 + j,
+                                U.b, fb);
                     if (hasy) tma_load_5d(st + xbytes, &tmdy, 16 * cog, -1, yl, U.z0 - 1 + j, U.b, fb);
                     if (++b == ns) { b = 0; ++use; }
                 }
@@ -991,29 +1037,6 @@ conv3d_wgrad_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
 // ------------------------------------------------------------------------ elementwise
 // Elementwise layer kernels on 8-channel (16-byte) chunks; every count and index fits in
 // 32 bits (mcx_denoiser_create bounds max_batch * nx * ny * nz * 96).
-struct Bf8 {
-    uint4 u;
-    __device__ void to(float *f) const
-    {
-        const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 t = __bfloat1622float2(h[i]);
-            f[2 * i] = t.x;
-            f[2 * i + 1] = t.y;
-        }
-    }
-    __device__ static Bf8 from(const float *f)
-    {
-        Bf8 r;
-        r.u.x = pack_bf16(f[0], f[1]);
-        r.u.y = pack_bf16(f[2], f[3]);
-        r.u.z = pack_bf16(f[4], f[5]);
-        r.u.w = pack_bf16(f[6], f[7]);
-        return r;
-    }
-};
-
 __device__ __forceinline__ uint4 ld16(const bf16 *p) { return *reinterpret_cast<const uint4 *>(p); }
 __device__ __forceinline__ void st16(bf16 *p, uint4 v) { *reinterpret_cast<uint4 *>(p) = v; }
 
@@ -1253,30 +1276,15 @@ __global__ void avgpool_fwd(const bf16 *X, Vol vo, int c, bf16 *Y)
     }
 }
 
-// nearest x2 upsampling of X (coarse, cx channels) into channels [0, cx) of the fine
-// volume vf, and the skip S (cs channels) into channels [cx, cx + cs)
-__global__ void upcat_fwd(const bf16 *X, int cx, const bf16 *S, int cs, Vol vf, bf16 *Y)
+// nearest x2 upsampling of X (coarse, c channels) to the fine volume vf.  The convolution
+// after it reads the skip channels from where the encoder left them (a second tensor map),
+// so they are not copied beside these
+__global__ void up_fwd(const bf16 *X, int c, Vol vf, bf16 *Y)
 {
-    const int c8 = (cx + cs) / 8, x8 = cx / 8, n = vf.n * vf.d * vf.h * vf.w * c8;
+    const int c8 = c / 8, n = vf.n * vf.d * vf.h * vf.w * c8;
     GRID_LOOP(i, n) {
         const int p = i / c8, j = i - p * c8;
-        const uint4 v = j < x8 ? ld16(X + (size_t)parent_of(p, vf) * cx + 8 * j)
-                               : ld16(S + (size_t)p * cs + 8 * (j - x8));
-        st16(Y + (size_t)p * (cx + cs) + 8 * j, v);
-    }
-}
-
-// head: out[p] = x[p] + hb + sum_c hw[c] Y[p][c]
-__global__ void head_fwd(const bf16 *Y, const float *x, const float *hw, const float *hb, int npos, float *out)
-{
-    GRID_LOOP(p, npos) {
-        float y[16];
-        Bf8{ld16(Y + 16 * (size_t)p)}.to(y);
-        Bf8{ld16(Y + 16 * (size_t)p + 8)}.to(y + 8);
-        float s = hb[0];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) s += hw[c] * y[c];
-        out[p] = x[p] + s;
+        st16(Y + 8 * (size_t)i, ld16(X + (size_t)parent_of(p, vf) * c + 8 * j));
     }
 }
 
@@ -1453,25 +1461,41 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
+// A convolution's input: cin channels of a, or cin - cb of a followed by cb of b (a skip
+// connection's, read where they are).
+struct Input {
+    const bf16 *a, *b;
+    int cb;
+    Input(const bf16 *a_, const bf16 *b_ = nullptr, int cb_ = 0) : a(a_), b(b_), cb(cb_) {}
+};
+
+// tensor map of windows: 16-channel boxes of whole padded lines (from x = -1) of activations
+// [n][d][h][w][c], in the 32-byte swizzle
+bool map_windows(CUtensorMap *m, const bf16 *ptr, int c, Vol v, int lines)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+    const cuuint32_t one[5] = {1, 1, 1, 1, 1};
+    const cuuint64_t dim[5] = {(cuuint64_t)c, (cuuint64_t)v.w, (cuuint64_t)v.h, (cuuint64_t)v.d, (cuuint64_t)v.n};
+    const cuuint64_t str[4] = {(cuuint64_t)c * 2, (cuuint64_t)v.w * c * 2, (cuuint64_t)v.h * v.w * c * 2,
+                               (cuuint64_t)v.d * v.h * v.w * c * 2};
+    const cuuint32_t box[5] = {16, (cuuint32_t)(v.w + 2), (cuuint32_t)lines, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(ptr), dim, str, box, one,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int CIN, int COUT>
-cudaError_t launch_tc_t(const bf16 *X, const bf16 *W, const float *bias, Vol v, int relu, bf16 *Y,
-                        unsigned *err, cudaStream_t st)
+cudaError_t launch_tc_t(const Input &X, const bf16 *W, const float *bias, Vol v, int relu, bf16 *Y,
+                        const Head &head, unsigned *err, cudaStream_t st)
 {
     constexpr int cin = CIN;
     if (v.w + 2 > 256 || tc_lines(v.w) > 256) return cudaErrorInvalidValue;
-    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (!enc) return cudaErrorNotSupported;
-    // activations [n][d][h][w][cin] as a 5-D tensor, innermost first
-    CUtensorMap mx;
-    const cuuint64_t xdim[5] = {(cuuint64_t)cin, (cuuint64_t)v.w, (cuuint64_t)v.h, (cuuint64_t)v.d, (cuuint64_t)v.n};
-    const cuuint64_t xstr[4] = {(cuuint64_t)cin * 2, (cuuint64_t)v.w * cin * 2, (cuuint64_t)v.h * v.w * cin * 2,
-                                (cuuint64_t)v.d * v.h * v.w * cin * 2};
-    const cuuint32_t xbox[5] = {16, (cuuint32_t)(v.w + 2), (cuuint32_t)tc_lines(v.w), 1, 1};
-    const cuuint32_t one[5] = {1, 1, 1, 1, 1};
-    if (enc(&mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(X), xdim, xstr, xbox, one,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
+    if (!tensor_map_encoder()) return cudaErrorNotSupported;
+    const int ca = cin - X.cb, g1 = ca / 16;
+    CUtensorMap mx, mx2;
+    if (!map_windows(&mx, X.a, ca, v, tc_lines(v.w))) return cudaErrorInvalidValue;
+    mx2 = mx;
+    if (X.cb && !map_windows(&mx2, X.b, X.cb, v, tc_lines(v.w))) return cudaErrorInvalidValue;
     if constexpr (!tc_wall(CIN, COUT)) {
         // weights too large to keep: the weights-stationary kernel, one CTA per SM (its
         // two units of accumulators take the SM's 512 tensor-memory columns)
@@ -1495,7 +1519,7 @@ cudaError_t launch_tc_t(const bf16 *X, const bf16 *W, const float *bias, Vol v, 
         }
         const long long wunits = (wtiles + tu - 1) / tu;
         const unsigned wblocks = (unsigned)std::max<long long>(1, std::min<long long>(wunits, wsms));
-        conv3d_fwd_ws<CIN, COUT><<<wblocks, kWsThreads, wsmem, st>>>(mx, W, bias, v, relu, Y, err, wns, tu);
+        conv3d_fwd_ws<CIN, COUT><<<wblocks, kWsThreads, wsmem, st>>>(mx, mx2, g1, W, bias, v, relu, Y, err, wns, tu);
         return cudaGetLastError();
     } else {
         const int ns = tc_stages(cin, COUT, v.w);
@@ -1529,17 +1553,17 @@ cudaError_t launch_tc_t(const bf16 *X, const bf16 *W, const float *bias, Vol v, 
         }
         const long long units = (long long)v.n * ((v.d + zc - 1) / zc) * tiles_plane;
         const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>(units, (long long)sms * per_sm));
-        conv3d_fwd_tc<CIN, COUT><<<blocks, kTcThreads, smem, st>>>(mx, W, bias, v, relu, Y, err, ns, zc);
+        conv3d_fwd_tc<CIN, COUT><<<blocks, kTcThreads, smem, st>>>(mx, mx2, g1, W, bias, v, relu, Y, err, ns, zc, head);
         return cudaGetLastError();
     }
 }
 
-cudaError_t launch_fwd_tc(const bf16 *X, int cin, const bf16 *W, const float *bias, Vol v, int cout,
-                          int relu, bf16 *Y, unsigned *err, cudaStream_t st)
+cudaError_t launch_fwd_tc(const Input &X, int cin, const bf16 *W, const float *bias, Vol v, int cout,
+                          int relu, bf16 *Y, unsigned *err, cudaStream_t st, const Head &head = Head{})
 {
     // the (cin, cout) pairs of the network's convolutions and of their input gradients
 #define MCX_TC(ci, co) \
-    if (cin == ci && cout == co) return launch_tc_t<ci, co>(X, W, bias, v, relu, Y, err, st);
+    if (cin == ci && cout == co) return launch_tc_t<ci, co>(X, W, bias, v, relu, Y, head, err, st);
     MCX_TC(16, 16) MCX_TC(16, 32) MCX_TC(16, 48) MCX_TC(32, 16) MCX_TC(32, 32) MCX_TC(32, 64)
     MCX_TC(32, 96) MCX_TC(48, 16) MCX_TC(64, 32) MCX_TC(64, 64) MCX_TC(96, 32)
 #undef MCX_TC
@@ -1547,24 +1571,16 @@ cudaError_t launch_fwd_tc(const bf16 *X, int cin, const bf16 *W, const float *bi
 }
 
 template <int CIN, int COUT>
-cudaError_t launch_wt_t(const bf16 *X, const bf16 *dY, Vol v, float *dW, unsigned *err, cudaStream_t st)
+cudaError_t launch_wt_t(const Input &X, const bf16 *dY, Vol v, float *dW, unsigned *err, cudaStream_t st)
 {
     if (v.w + 2 > 256 || wt_ylines(v.w) > 256) return cudaErrorInvalidValue;
-    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (!enc) return cudaErrorNotSupported;
-    // 16-channel boxes of whole padded lines (from x = -1), 32-byte swizzle
-    CUtensorMap mx, my;
-    const cuuint32_t one[5] = {1, 1, 1, 1, 1};
-    auto map5 = [&](CUtensorMap *m, const bf16 *ptr, int c, int lines) {
-        const cuuint64_t dim[5] = {(cuuint64_t)c, (cuuint64_t)v.w, (cuuint64_t)v.h, (cuuint64_t)v.d, (cuuint64_t)v.n};
-        const cuuint64_t str[4] = {(cuuint64_t)c * 2, (cuuint64_t)v.w * c * 2, (cuuint64_t)v.h * v.w * c * 2,
-                                   (cuuint64_t)v.d * v.h * v.w * c * 2};
-        const cuuint32_t box[5] = {16, (cuuint32_t)(v.w + 2), (cuuint32_t)lines, 1, 1};
-        return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(ptr), dim, str, box, one,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    };
-    if (!map5(&mx, X, CIN, wt_xlines(v.w)) || !map5(&my, dY, COUT, wt_ylines(v.w))) return cudaErrorInvalidValue;
+    if (!tensor_map_encoder()) return cudaErrorNotSupported;
+    const int ca = CIN - X.cb, g1 = ca / 16;
+    CUtensorMap mx, mx2, my;
+    if (!map_windows(&mx, X.a, ca, v, wt_xlines(v.w)) || !map_windows(&my, dY, COUT, v, wt_ylines(v.w)))
+        return cudaErrorInvalidValue;
+    mx2 = mx;
+    if (X.cb && !map_windows(&mx2, X.b, X.cb, v, wt_xlines(v.w))) return cudaErrorInvalidValue;
     const int ns = wt_stages(v.w);
     if (ns < 2) return cudaErrorInvalidValue;
     const int smem = wt_smem_bytes(v.w, ns);
@@ -1590,13 +1606,13 @@ cudaError_t launch_wt_t(const bf16 *X, const bf16 *dY, Vol v, float *dW, unsigne
     const long long units = (long long)v.n * ((v.d + zc - 1) / zc) * tiles_plane;
     const long long per_pair = std::max<long long>(1, std::min<long long>(units, std::max<long long>(1, slots / pairs)));
     const dim3 grid((unsigned)per_pair, (unsigned)pairs);
-    conv3d_wgrad_tc<CIN, COUT><<<grid, kWtThreads, smem, st>>>(mx, my, v, ns, zc, dW, err);
+    conv3d_wgrad_tc<CIN, COUT><<<grid, kWtThreads, smem, st>>>(mx, mx2, g1, my, v, ns, zc, dW, err);
     return cudaGetLastError();
 }
 
 // dW (FP32, [27][cout][cin]) += the weight gradient of a convolution with input X and
 // output gradient dY; (cin, cout) one of the network's layer pairs
-cudaError_t launch_bwd_w(const bf16 *X, int cin, const bf16 *dY, int cout, Vol v, float *dW, unsigned *err,
+cudaError_t launch_bwd_w(const Input &X, int cin, const bf16 *dY, int cout, Vol v, float *dW, unsigned *err,
                          cudaStream_t st)
 {
 #define MCX_WG(ci, co) \
@@ -1692,13 +1708,15 @@ static mcx_status refresh_weights(mcx_denoiser *d, cudaStream_t st)
 }
 
 // forward pass for n volumes; activations stay for the backward pass
-static mcx_status forward(mcx_denoiser *d, const float *x, const float *aux, int n, float *out, cudaStream_t st)
+// (keep: the last layer's too, which otherwise only forms the output)
+static mcx_status forward(mcx_denoiser *d, const float *x, const float *aux, int n, float *out, bool keep,
+                          cudaStream_t st)
 {
     const Vol v0 = level_vol(d, 0, n), v1 = level_vol(d, 1, n), v2 = level_vol(d, 2, n);
     const float *P = d->params.as<float>();
-    auto conv = [&](int l, const bf16 *in, Vol v) {
-        return launch_fwd_tc(in, kLayers[l].cin, d->wf[l].as<bf16>(), P + d->b_off[l], v,
-                             kLayers[l].cout, 1, d->a[l].as<bf16>(), d->status.as<unsigned>(), st);
+    auto conv = [&](int l, const Input &in, Vol v, bool store = true, const Head &head = Head{}) {
+        return launch_fwd_tc(in, kLayers[l].cin, d->wf[l].as<bf16>(), P + d->b_off[l], v, kLayers[l].cout, 1,
+                             store ? d->a[l].as<bf16>() : nullptr, d->status.as<unsigned>(), st, head);
     };
     if (d->n_aux == 0 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
         // one input channel: the direct input layer, which reads the input in 16-byte
@@ -1719,14 +1737,12 @@ static mcx_status forward(mcx_denoiser *d, const float *x, const float *aux, int
     avgpool_fwd<<<grid1(v2.pos() * 4), 256, 0, st>>>(d->a[3].as<bf16>(), v2, 32, d->p2.as<bf16>());
     DNC(d, conv(4, d->p2.as<bf16>(), v2), "conv ba");
     DNC(d, conv(5, d->a[4].as<bf16>(), v2), "conv bb");
-    upcat_fwd<<<grid1(v1.pos() * 12), 256, 0, st>>>(d->a[5].as<bf16>(), 64, d->a[3].as<bf16>(), 32, v1, d->u2.as<bf16>());
-    DNC(d, conv(6, d->u2.as<bf16>(), v1), "conv d2a");
+    up_fwd<<<grid1(v1.pos() * 8), 256, 0, st>>>(d->a[5].as<bf16>(), 64, v1, d->u2.as<bf16>());
+    DNC(d, conv(6, Input(d->u2.as<bf16>(), d->a[3].as<bf16>(), 32), v1), "conv d2a");
     DNC(d, conv(7, d->a[6].as<bf16>(), v1), "conv d2b");
-    upcat_fwd<<<grid1(v0.pos() * 6), 256, 0, st>>>(d->a[7].as<bf16>(), 32, d->a[1].as<bf16>(), 16, v0, d->u1.as<bf16>());
-    DNC(d, conv(8, d->u1.as<bf16>(), v0), "conv d1a");
-    DNC(d, conv(9, d->a[8].as<bf16>(), v0), "conv d1b");
-    head_fwd<<<grid1(v0.pos()), 256, 0, st>>>(d->a[9].as<bf16>(), x, P + d->hw_off, P + d->hb_off,
-                                             (int)v0.pos(), out);
+    up_fwd<<<grid1(v0.pos() * 4), 256, 0, st>>>(d->a[7].as<bf16>(), 32, v0, d->u1.as<bf16>());
+    DNC(d, conv(8, Input(d->u1.as<bf16>(), d->a[1].as<bf16>(), 16), v0), "conv d1a");
+    DNC(d, conv(9, d->a[8].as<bf16>(), v0, keep, Head{P + d->hw_off, P + d->hb_off, x, out}), "conv d1b");
     DNC(d, cudaGetLastError(), "forward");
     return MCX_OK;
 }
@@ -1751,7 +1767,7 @@ static mcx_status relu_bwd(mcx_denoiser *d, int l, Vol v, int src, GradSource S,
 
 // backward of a conv layer l with input `in`: dA (gradient of its output before the ReLU, in
 // ga[l]) -> weight gradient, and (if dIn) the input gradient
-static mcx_status conv_bwd(mcx_denoiser *d, int l, const bf16 *in, Vol v, bf16 *dIn, cudaStream_t st)
+static mcx_status conv_bwd(mcx_denoiser *d, int l, const Input &in, Vol v, bf16 *dIn, cudaStream_t st)
 {
     const LayerSpec &L = kLayers[l];
     float *G = d->grads.as<float>();
@@ -1780,12 +1796,12 @@ static mcx_status backward(mcx_denoiser *d, const float *x, const float *target,
 #define MCX_RELU(l, v, src, S) if ((s = relu_bwd(d, l, v, src, S, st)) != MCX_OK) return s
     if ((s = conv_bwd(d, 9, d->a[8].as<bf16>(), v0, d->ga[8].as<bf16>(), st)) != MCX_OK) return s;
     MCX_RELU(8, v0, kGradPlain, none);
-    if ((s = conv_bwd(d, 8, d->u1.as<bf16>(), v0, d->gu1.as<bf16>(), st)) != MCX_OK) return s;
+    if ((s = conv_bwd(d, 8, Input(d->u1.as<bf16>(), d->a[1].as<bf16>(), 16), v0, d->gu1.as<bf16>(), st)) != MCX_OK) return s;
     // upcat 1: coarse part -> d2b's output, skip part -> e1b's output (later)
     MCX_RELU(7, v1, kGradUp, up1);
     if ((s = conv_bwd(d, 7, d->a[6].as<bf16>(), v1, d->ga[6].as<bf16>(), st)) != MCX_OK) return s;
     MCX_RELU(6, v1, kGradPlain, none);
-    if ((s = conv_bwd(d, 6, d->u2.as<bf16>(), v1, d->gu2.as<bf16>(), st)) != MCX_OK) return s;
+    if ((s = conv_bwd(d, 6, Input(d->u2.as<bf16>(), d->a[3].as<bf16>(), 32), v1, d->gu2.as<bf16>(), st)) != MCX_OK) return s;
     MCX_RELU(5, v2, kGradUp, up2);
     if ((s = conv_bwd(d, 5, d->a[4].as<bf16>(), v2, d->ga[4].as<bf16>(), st)) != MCX_OK) return s;
     MCX_RELU(4, v2, kGradPlain, none);
@@ -1859,7 +1875,7 @@ mcx_status mcx_denoiser_create(mcx_denoiser **out, uint32_t nx, uint32_t ny, uin
         A(d->ga[l], np * kLayers[l].cout * B2);
     }
     A(d->x16, p0 * 16 * B2); A(d->p1, p1 * 16 * B2); A(d->p2, p2 * 32 * B2);
-    A(d->u2, p1 * 96 * B2); A(d->u1, p0 * 48 * B2); A(d->out, p0 * 4); A(d->loss, 4);
+    A(d->u2, p1 * 64 * B2); A(d->u1, p0 * 32 * B2); A(d->out, p0 * 4); A(d->loss, 4);
     A(d->xin, p0 * 4);
     A(d->status, 4);
     A(d->gp1, p1 * 16 * B2); A(d->gp2, p2 * 32 * B2); A(d->gu2, p1 * 96 * B2); A(d->gu1, p0 * 48 * B2);
@@ -1917,7 +1933,11 @@ mcx_status mcx_denoiser_forward(mcx_denoiser *d, const float *x_dev, const float
     if (!d || !x_dev || !y_dev || (d->n_aux && !aux_dev)) return dn_fail(d, MCX_E_ARG, "NULL argument");
     if (n < 1 || (int)n > d->maxb) return dn_fail(d, MCX_E_ARG, "n must be 1..max_batch");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    mcx_status s = forward(d, x_dev, aux_dev, (int)n, d->out.as<float>(), st);
+    // straight into y_dev, unless it overlaps the input elsewhere than element on element
+    const size_t count = (size_t)level_vol(d, 0, n).pos();
+    if (y_dev == x_dev || y_dev + count <= x_dev || x_dev + count <= y_dev)
+        return forward(d, x_dev, aux_dev, (int)n, y_dev, false, st);
+    mcx_status s = forward(d, x_dev, aux_dev, (int)n, d->out.as<float>(), false, st);
     if (s != MCX_OK) return s;
     DNC(d, cudaMemcpyAsync(y_dev, d->out.p, (size_t)level_vol(d, 0, n).pos() * 4, cudaMemcpyDeviceToDevice, st),
         "copying the output");
@@ -1930,7 +1950,7 @@ mcx_status mcx_denoiser_train_step(mcx_denoiser *d, const float *x_dev, const fl
     if (!d || !x_dev || !t_dev || (d->n_aux && !aux_dev)) return dn_fail(d, MCX_E_ARG, "NULL argument");
     if (n < 1 || (int)n > d->maxb) return dn_fail(d, MCX_E_ARG, "n must be 1..max_batch");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    mcx_status s = forward(d, x_dev, aux_dev, (int)n, d->out.as<float>(), st);
+    mcx_status s = forward(d, x_dev, aux_dev, (int)n, d->out.as<float>(), true, st);
     if (s != MCX_OK) return s;
     if ((s = backward(d, x_dev, t_dev, (int)n, st)) != MCX_OK) return s;
     if (lr > 0.f) {
@@ -1991,7 +2011,7 @@ mcx_status mcx_denoiser_apply(mcx_denoiser *d, const float *phi_in_dev, const fl
     const long long cnt = level_vol(d, 0, (int)n).pos();
     encode_kernel<<<grid1(cnt), 256, 0, st>>>(phi_in_dev, cnt, d->floor_, d->mu, 1.f / d->sigma, d->xin.as<float>());
     DNC(d, cudaGetLastError(), "encode");
-    mcx_status s = forward(d, d->xin.as<float>(), aux_dev, (int)n, d->out.as<float>(), st);
+    mcx_status s = forward(d, d->xin.as<float>(), aux_dev, (int)n, d->out.as<float>(), false, st);
     if (s != MCX_OK) return s;
     decode_kernel<<<grid1(cnt), 256, 0, st>>>(d->out.as<float>(), cnt, d->floor_, d->mu, d->sigma, phi_out_dev);
     DNC(d, cudaGetLastError(), "decode");
