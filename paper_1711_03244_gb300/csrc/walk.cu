@@ -1008,8 +1008,12 @@ template <typename R, bool DET, int ACC, bool ST, bool BATCH = false, bool PAD =
 cudaError_t shape_for(int block, int n_media, int n_det, int tile_e, LaunchShape *shape)
 {
     const size_t smem = SmemLayout<R>(n_media, DET ? n_det : 0, tile_e).total;
+    // the kernel's limit holds for every handle, so it is the most that any run asks for: a
+    // handle keeps its shape, and must still launch after another one with fewer media
+    const size_t most = SmemLayout<R>(kMaxMedia, DET ? kMaxDet : 0,
+                                      ACC == kAccCompensated ? kTileMaxEntries : 0).total;
     cudaError_t e = cudaFuncSetAttribute(walk_kernel<R, DET, ACC, ST, BATCH, PAD, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
