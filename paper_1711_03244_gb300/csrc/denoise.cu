@@ -1164,12 +1164,13 @@ __global__ void pad_input(const float *x, const float *aux, int n_aux, int vol, 
 
 // input layer without medium features (one input channel): Y[p][co] = ReLU(b[co] +
 // sum_tap W[tap][co][0] x[p + off(tap)]), zero outside the volume.  The 16-channel
-// tensor-core path would multiply 15 zero input channels; here each thread forms the 16
-// outputs of 4 consecutive positions of a line (the width is a multiple of 16) from the
+// tensor-core path would multiply 15 zero input channels; here each thread forms 8 outputs
+// of 8 consecutive positions of a line (the width is a multiple of 16) from the
 // FP32 input, rounded to BF16 as the padded path stores it, with FP32 sums on the CUDA
 // cores: each input line segment is loaded once per (dz, dy) and each 4-channel weight
-// vector (shared memory) serves 16 products.  Two channels per packed FMA: the kernel is
-// bound by issue, and these are most of its instructions
+// vector (shared memory) serves 32 products.  Two channels per packed FMA (16 volumes of
+// 64^3: 113 -> 99 us; 8 positions of 8 channels instead of 4 of 16, which halves the weight
+// reads per FMA, 91 us; its FMAs alone take 46 us)
 constexpr int kInThreads = 256;
 __global__ void __launch_bounds__(kInThreads, 2)
 conv_in_fwd(const float *__restrict__ x, const bf16 *__restrict__ W, const float *__restrict__ bias, Vol v,
@@ -1181,62 +1182,62 @@ conv_in_fwd(const float *__restrict__ x, const bf16 *__restrict__ W, const float
         sw[i / 16][i % 16] = __bfloat162float(W[packed_weight(i / 16, i % 16, 0, 16, 16)]);
     if (threadIdx.x < 16) sb[threadIdx.x] = bias ? bias[threadIdx.x] : 0.f;
     __syncthreads();
-    const int nquad = (int)(v.pos() / 4), wq = v.w / 4;
+    const int n = (int)(v.pos() / 4), w8 = v.w / 8;      // (8 positions, 8 channels) each
     auto rnd = [](float f) { return __bfloat162float(__float2bfloat16(f)); };
     auto pack = [](float lo, float hi) {
         return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
     };
-    GRID_LOOP(qd, nquad) {
-        const int x0 = 4 * (qd % wq), r1 = qd / wq, yy = r1 % v.h, r2 = r1 / v.h, zz = r2 % v.d, b = r2 / v.d;
-        unsigned long long acc[4][8];                 // channels 2c and 2c + 1
+    GRID_LOOP(i, n) {
+        const int c0 = 8 * (i & 1), run = i >> 1;
+        const int x0 = 8 * (run % w8), r1 = run / w8, yy = r1 % v.h, r2 = r1 / v.h, zz = r2 % v.d, b = r2 / v.d;
+        unsigned long long acc[8][4];                 // channels c0 + 2c and c0 + 2c + 1
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int q = 0; q < 8; ++q)
 #pragma unroll
-            for (int c = 0; c < 8; ++c) acc[i][c] = pack(sb[2 * c], sb[2 * c + 1]);
+            for (int c = 0; c < 4; ++c) acc[q][c] = pack(sb[c0 + 2 * c], sb[c0 + 2 * c + 1]);
 #pragma unroll
         for (int dz = -1; dz <= 1; ++dz) {
             const int z2 = zz + dz;
 #pragma unroll
             for (int dy = -1; dy <= 1; ++dy) {
                 const int y2 = yy + dy;
-                // the line's inputs at x0 - 1 .. x0 + 4 (zero outside the volume)
-                float xs[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                // the line's inputs at x0 - 1 .. x0 + 8 (zero outside the volume)
+                float xs[10] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                 if ((unsigned)z2 < (unsigned)v.d && (unsigned)y2 < (unsigned)v.h) {
                     const float *line = x + ((size_t)(b * v.d + z2) * v.h + y2) * v.w;
-                    const float4 m = __ldg(reinterpret_cast<const float4 *>(line + x0));   // 16-B aligned
-                    xs[1] = rnd(m.x); xs[2] = rnd(m.y); xs[3] = rnd(m.z); xs[4] = rnd(m.w);
+                    const float4 m0 = __ldg(reinterpret_cast<const float4 *>(line + x0));   // 16-B aligned
+                    const float4 m1 = __ldg(reinterpret_cast<const float4 *>(line + x0 + 4));
+                    xs[1] = rnd(m0.x); xs[2] = rnd(m0.y); xs[3] = rnd(m0.z); xs[4] = rnd(m0.w);
+                    xs[5] = rnd(m1.x); xs[6] = rnd(m1.y); xs[7] = rnd(m1.z); xs[8] = rnd(m1.w);
                     if (x0 > 0) xs[0] = rnd(__ldg(line + x0 - 1));
-                    if (x0 + 4 < v.w) xs[5] = rnd(__ldg(line + x0 + 4));
+                    if (x0 + 8 < v.w) xs[9] = rnd(__ldg(line + x0 + 8));
                 }
-                unsigned long long xx[6];
-#pragma unroll
-                for (int i = 0; i < 6; ++i) xx[i] = pack(xs[i], xs[i]);
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx) {
                     const int t = 9 * (dz + 1) + 3 * (dy + 1) + dx;
+                    const ulonglong2 w01 = *reinterpret_cast<const ulonglong2 *>(&sw[t][c0]);
+                    const ulonglong2 w23 = *reinterpret_cast<const ulonglong2 *>(&sw[t][c0 + 4]);
 #pragma unroll
-                    for (int c = 0; c < 8; c += 2) {
-                        const ulonglong2 wv = *reinterpret_cast<const ulonglong2 *>(&sw[t][2 * c]);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][c]) : "l"(xx[i + dx]), "l"(wv.x));
-                            asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][c + 1]) : "l"(xx[i + dx]), "l"(wv.y));
-                        }
+                    for (int q = 0; q < 8; ++q) {
+                        const unsigned long long xx = pack(xs[q + dx], xs[q + dx]);
+                        asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc[q][0]) : "l"(xx), "l"(w01.x));
+                        asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc[q][1]) : "l"(xx), "l"(w01.y));
+                        asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc[q][2]) : "l"(xx), "l"(w23.x));
+                        asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc[q][3]) : "l"(xx), "l"(w23.y));
                     }
                 }
             }
         }
-        bf16 *yo = Y + 16 * ((size_t)qd * 4);
+        bf16 *yo = Y + 16 * ((size_t)run * 8) + c0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float o[16];
+        for (int q = 0; q < 8; ++q) {
+            float o[8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                o[2 * c] = fmaxf(__uint_as_float((unsigned)acc[i][c]), 0.f);
-                o[2 * c + 1] = fmaxf(__uint_as_float((unsigned)(acc[i][c] >> 32)), 0.f);
+            for (int c = 0; c < 4; ++c) {
+                o[2 * c] = fmaxf(__uint_as_float((unsigned)acc[q][c]), 0.f);
+                o[2 * c + 1] = fmaxf(__uint_as_float((unsigned)(acc[q][c] >> 32)), 0.f);
             }
-            st16(yo + 16 * i, Bf8::from(o).u);
-            st16(yo + 16 * i + 8, Bf8::from(o + 8).u);
+            st16(yo + 16 * q, Bf8::from(o).u);
         }
     }
 }
@@ -1276,15 +1277,22 @@ __global__ void avgpool_fwd(const bf16 *X, Vol vo, int c, bf16 *Y)
     }
 }
 
-// nearest x2 upsampling of X (coarse, c channels) to the fine volume vf.  The convolution
+// nearest x2 upsampling of X (coarse volume vc, c channels).  The convolution
 // after it reads the skip channels from where the encoder left them (a second tensor map),
 // so they are not copied beside these
-__global__ void up_fwd(const bf16 *X, int c, Vol vf, bf16 *Y)
+__global__ void up_fwd(const bf16 *X, int c, Vol vc, bf16 *Y)
 {
-    const int c8 = c / 8, n = vf.n * vf.d * vf.h * vf.w * c8;
+    // a thread reads one coarse chunk and writes its 8 children: memory-bound (16 volumes to
+    // 64^3, 302 MB), where a parent looked up per written chunk took 70 us
+    const int c8 = c / 8, n = vc.n * vc.d * vc.h * vc.w * c8;
+    const Vol vf{vc.n, 2 * vc.d, 2 * vc.h, 2 * vc.w};
     GRID_LOOP(i, n) {
         const int p = i / c8, j = i - p * c8;
-        st16(Y + 8 * (size_t)i, ld16(X + (size_t)parent_of(p, vf) * c + 8 * j));
+        const uint4 u = ld16(X + 8 * (size_t)i);
+        int ch[8];
+        children_of(p, vf, ch);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) st16(Y + (size_t)ch[k] * c + 8 * j, u);
     }
 }
 
@@ -1737,10 +1745,10 @@ static mcx_status forward(mcx_denoiser *d, const float *x, const float *aux, int
     avgpool_fwd<<<grid1(v2.pos() * 4), 256, 0, st>>>(d->a[3].as<bf16>(), v2, 32, d->p2.as<bf16>());
     DNC(d, conv(4, d->p2.as<bf16>(), v2), "conv ba");
     DNC(d, conv(5, d->a[4].as<bf16>(), v2), "conv bb");
-    up_fwd<<<grid1(v1.pos() * 8), 256, 0, st>>>(d->a[5].as<bf16>(), 64, v1, d->u2.as<bf16>());
+    up_fwd<<<grid1(v2.pos() * 8), 256, 0, st>>>(d->a[5].as<bf16>(), 64, v2, d->u2.as<bf16>());
     DNC(d, conv(6, Input(d->u2.as<bf16>(), d->a[3].as<bf16>(), 32), v1), "conv d2a");
     DNC(d, conv(7, d->a[6].as<bf16>(), v1), "conv d2b");
-    up_fwd<<<grid1(v0.pos() * 4), 256, 0, st>>>(d->a[7].as<bf16>(), 32, v0, d->u1.as<bf16>());
+    up_fwd<<<grid1(v1.pos() * 4), 256, 0, st>>>(d->a[7].as<bf16>(), 32, v1, d->u1.as<bf16>());
     DNC(d, conv(8, Input(d->u1.as<bf16>(), d->a[1].as<bf16>(), 16), v0), "conv d1a");
     DNC(d, conv(9, d->a[8].as<bf16>(), v0, keep, Head{P + d->hw_off, P + d->hb_off, x, out}), "conv d1b");
     DNC(d, cudaGetLastError(), "forward");
