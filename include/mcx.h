@@ -100,7 +100,8 @@ typedef struct mcx_run_cfg {
                                          mode 0 loses up to tens of percent in the hottest
                                          voxels, where additions fall below half an ulp) */
     int32_t block_size;            /* threads per block, multiple of 32 (0 = 256) */
-    int32_t grid_size;             /* persistent blocks (0 = SMs x resident blocks/SM) */
+    int32_t grid_size;             /* persistent blocks (0 = by the photon count, at most SMs x
+                                      resident blocks/SM) */
     int32_t precision;             /* 0: FP32 photon state (the product path); 1: the same walk
                                       in FP64, a trajectory-parity diagnostic that runs at the
                                       part's much lower FP64 rate */
@@ -261,7 +262,7 @@ typedef struct mcx_batch_cfg {
     int32_t accum_mode;            /* 0 (FP32 atomics) or 2 (FP64 atomics, default) */
     int32_t block_size;            /* 0 = 256 (multiple of 32, <= 256) */
     int32_t claim_chunk;           /* photon ids per warp claim: 0 = 32; 32..4096 */
-    int32_t grid_size;             /* 0 = SMs x resident blocks per SM */
+    int32_t grid_size;             /* 0 = by the photon count, as in mcx_run_cfg */
     uint64_t max_events_per_photon;/* 0 = 1e8 */
     int32_t use_graph;             /* 1: record the run (zeroing, walk, reductions) as a CUDA
                                       graph on first use and replay it while the batch and the

@@ -446,6 +446,11 @@ mcx_status mcx_batch_run(mcx_batch *b, const mcx_batch_cfg *cfg)
         if (st != MCX_OK) return st;
         b->dirty = false;
     }
+    if (cfg->grid_size == 0) {
+        uint64_t photons = 0;
+        for (const SimHost *sim : b->sims) photons += sim->n_photons;
+        shape = walk_grid(shape, photons);
+    }
     BCUDA(b, cudaEventRecord(b->ev0, stream), "recording an event");
     if (cfg->use_graph) {
         if (!b->graph) {

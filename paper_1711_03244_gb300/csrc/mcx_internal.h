@@ -113,7 +113,38 @@ struct WalkParams {
 
 struct LaunchShape {
     int grid, block, blocks_per_sm, regs;
+    int warps;                        // warps per block that take photons; 0: as the launch finds
 };
+
+// The grid of a run of n photons whose caller gives none: as many warps per SM as the run
+// keeps busy.  A run ends with its longest histories, and in that time every resident warp
+// still issues the walk for the few lanes it has left; fewer warps take more photons each,
+// stay full for longer and iterate faster.  Too few leave the issue slots idle.  So 4 warps
+// per SM (one per scheduler) up to 2.6 photons per lane, 8 up to 3.5, 16 up to 6.5, 24 up
+// to 13, then all 32.  Measured kernel times, ms, at 32 / 24 / 16 / 8 / 4 warps per SM:
+//   cube        2e4  4.23 /  4.22 /  3.93 /  3.93 /  3.75    1e5   7.41 /  6.82 /  5.40 /  4.62 /  5.41
+//               3e5  9.73 /  7.93 /  6.61 /  7.57 / 10.9     1e6  14.0  / 13.2  / 13.2  / 17.6
+//               1e7  81.0 / 83.0  / 94.7
+//   B2a         1e5  2.96 /  2.78 /  2.58 /  2.57 /  2.83    3e5   4.07 /  3.53 /  3.16 /  3.58
+//               1e6  5.91 /  5.36 /  5.52                    1e7  29.3  / 30.8  / 36.7
+//   layers      3e5  6.59 /  5.90 /  6.28 /  8.28            1e6  12.3  / 12.1  / 13.9
+//   ellipsoids (96 mm, mus about 19/mm) 5e5  17.9 / 14.3 / 11.1 / 9.96 / 13.0
+inline LaunchShape walk_grid(LaunchShape s, unsigned long long n)
+{
+    if (s.blocks_per_sm < 1) return s;
+    const int wpb = s.block / 32, most = s.blocks_per_sm * wpb;
+    const unsigned long long sms = (unsigned long long)(s.grid / s.blocks_per_sm), lane = 32 * sms;
+    int want = 4;
+    if (n > lane * 4 * 26 / 10) want = 8;
+    if (n > lane * 8 * 35 / 10) want = 16;
+    if (n > lane * 16 * 65 / 10) want = 24;
+    if (n > lane * 24 * 13) want = most;
+    if (want > most) want = most;
+    const int blocks = (want + wpb - 1) / wpb;
+    s.grid = (int)sms * blocks;
+    s.warps = (want + blocks - 1) / blocks;
+    return s;
+}
 
 // Walk precision: the FP32 product path, or the same kernel in FP64 (trajectory-parity
 // diagnostic; FP64 runs at a small fraction of the FP32 rate on this part).

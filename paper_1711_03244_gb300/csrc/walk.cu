@@ -35,11 +35,11 @@
 //    condition in its own branch and crossing every face at once: two spheres, 2e7 photons
 //    175.6 -> 147 ms; layered tissue, 1e7 photons 87.0 -> 83.2 ms; 24 uneven batched
 //    simulations 57.6 -> 48.8 ms; cube, 3e5 photons 12.8 -> 9.5 ms.
-//  * A run with fewer photons than the grid has lanes gives each block its share: as few
-//    warps as hold it.  Its time is that of the longest history, whose warp then neither
-//    waits for warps beside it nor sits on an SM that took most of the photons
-//    (cube, 2e3 / 2e4 / 5e4 / 1e5 photons: 3.5 / 4.5 / 6.3 / 8.2 -> 2.9 / 4.0 / 4.8 / 7.5 ms;
-//    spreading them over all warps, a few lanes each, was slower: 5.2 ms at 2e4).
+//  * A short run takes fewer warps per SM (walk_grid), and one with fewer photons than lanes
+//    shares them out evenly: its time is that of the longest history, whose warp should
+//    neither wait for warps beside it nor sit on an SM that took most of the photons
+//    (cube, 2e3 / 2e4 / 1e5 / 3e5 photons: 3.5 / 4.5 / 8.2 / 9.7 -> 2.9 / 3.7 / 4.6 / 6.6 ms;
+//    spread over all warps, a few lanes each: 5.2 ms at 2e4).
 //  * Fast hardware math (MUFU ex2/lg2/sin/cos/rsqrt/rcp) in the FP32 path, the CUDA
 //    analogue of the paper's "native" math optimisation; the same kernel instantiated in
 //    FP64 serves as the trajectory-parity diagnostic.
@@ -1028,19 +1028,22 @@ cudaError_t shape_for(int block, int n_media, int n_det, int tile_e, LaunchShape
     shape->blocks_per_sm = per_sm;
     shape->grid = sms * (per_sm > 0 ? per_sm : 1);
     shape->regs = fa.numRegs;
+    shape->warps = 0;
     return cudaSuccess;
 }
 
-// How a run's photons are shared out: all lanes and the caller's claim size, or, when there
-// are fewer photons than lanes, as few warps of each block as hold the block's share.
+// How a run's photons are shared out: the shape's warps, 32 lanes each, and the caller's
+// claim size; where there are fewer photons than those lanes, each of the shape's warps
+// takes its share in fewer lanes, or (a grid of the caller's) as few warps of each block as
+// hold the block's share.
 WalkParams shared_out(WalkParams p, const LaunchShape &s)
 {
     const unsigned wpb = (unsigned)s.block / 32u, grid = (unsigned)s.grid;
     p.lanes = 32;
-    p.warps = wpb;
-    if (p.claim_static || p.n_photons >= 32ull * wpb * grid) return p;
+    p.warps = s.warps > 0 ? (unsigned)s.warps : wpb;
+    if (p.claim_static || p.n_photons >= 32ull * p.warps * grid) return p;
     const unsigned per_block = p.n_photons ? ((unsigned)p.n_photons + grid - 1u) / grid : 1u;
-    p.warps = (per_block + 31u) / 32u;
+    if (s.warps <= 0) p.warps = (per_block + 31u) / 32u;
     p.lanes = (per_block + p.warps - 1u) / p.warps;
     p.claim_chunk = p.lanes;
     return p;

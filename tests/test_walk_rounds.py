@@ -41,6 +41,19 @@ def test_sharing_does_not_change_photons(g, reference, n, block, grid):
     assert balance(r["tally"]) == pytest.approx(n, rel=1e-6)
 
 
+# photon counts at which the grid changes (2.6, 3.5, 6.5 and 13 photons per lane of 4, 8, 16
+# and 24 warps on each of 152 SMs), each against the full grid
+@pytest.mark.parametrize("n", [50585, 50586, 136192, 136193, 505856, 505857, 1517568, 1517569])
+@pytest.mark.parametrize("block", [0, 128])
+def test_grid_by_photon_count(g, n, block):
+    wl = f32(workloads.c1(n_photons=n).with_(labels=np.ones((8, 8, 8), dtype=np.uint8), src_pos=(4.0, 4.0, 0.0)))
+    a = gpu_run(wl, exit_log=n, seed=9, block_size=block)
+    b = gpu_run(wl, exit_log=n, seed=9, block_size=block, grid_size=152 * (4 if block == 0 else 8))
+    assert a["stats"] == b["stats"] and a["stats"]["photons"] == n
+    assert np.array_equal(a["exits"], b["exits"])
+    assert np.allclose(a["energy"], b["energy"], rtol=1e-6)
+
+
 @pytest.mark.parametrize("case", ["gates", "limit", "cap", "roulette", "axial"])
 def test_rare_path_matches_oracle(g, case):
     import oracle as orc
