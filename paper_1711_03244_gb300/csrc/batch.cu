@@ -448,8 +448,12 @@ mcx_status mcx_batch_run(mcx_batch *b, const mcx_batch_cfg *cfg)
     }
     if (cfg->grid_size == 0) {
         uint64_t photons = 0;
-        for (const SimHost *sim : b->sims) photons += sim->n_photons;
-        shape = walk_grid(shape, photons);
+        double largest = 0;
+        for (const SimHost *sim : b->sims) {
+            photons += sim->n_photons;
+            largest = std::max(largest, (double)sim->nx * sim->ny * sim->nz * cfg->n_gates * sizeof(double));
+        }
+        shape = walk_grid(shape, photons, grid_limits(largest, true));
     }
     BCUDA(b, cudaEventRecord(b->ev0, stream), "recording an event");
     if (cfg->use_graph) {

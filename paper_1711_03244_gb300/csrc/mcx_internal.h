@@ -119,9 +119,19 @@ struct LaunchShape {
 // The grid of a run of n photons whose caller gives none: as many warps per SM as the run
 // keeps busy.  A run ends with its longest histories, and in that time every resident warp
 // still issues the walk for the few lanes it has left; fewer warps take more photons each,
-// stay full for longer and iterate faster.  Too few leave the issue slots idle.  So 4 warps
-// per SM (one per scheduler) up to 2.6 photons per lane, 8 up to 3.5, 16 up to 6.5, 24 up
-// to 13, then all 32.  Measured kernel times, ms, at 32 / 24 / 16 / 8 / 4 warps per SM:
+// stay full for longer and iterate faster.  Too few leave the issue slots idle, and sooner
+// where label loads and deposits go past L2.  So 4, 8, 16 and 24 warps per SM up to so many
+// photons per lane, then all 32: with a map that stays in L2, with a larger one, and for a
+// batch of such maps, whose histories differ most.
+constexpr double kGridSmallMap[4] = {2.6, 3.5, 13, 26}, kGridLargeMap[4] = {2.6, 3.5, 6.5, 13},
+                 kGridBatch[4] = {2.6, 10, 20, 34};
+constexpr double kGridMapBytes = 128e6;
+
+inline const double *grid_limits(double map_bytes, bool batch)
+{
+    return map_bytes > kGridMapBytes ? kGridLargeMap : batch ? kGridBatch : kGridSmallMap;
+}
+// Measured kernel times, ms, at 32 / 24 / 16 / 8 / 4 warps per SM:
 //   cube        2e4  4.23 /  4.22 /  3.93 /  3.93 /  3.75    1e5   7.41 /  6.82 /  5.40 /  4.62 /  5.41
 //               3e5  9.73 /  7.93 /  6.61 /  7.57 / 10.9     1e6  14.0  / 13.2  / 13.2  / 17.6
 //               1e7  81.0 / 83.0  / 94.7
@@ -129,19 +139,20 @@ struct LaunchShape {
 //               1e6  5.91 /  5.36 /  5.52                    1e7  29.3  / 30.8  / 36.7
 //   layers      3e5  6.59 /  5.90 /  6.28 /  8.28            1e6  12.3  / 12.1  / 13.9
 //   ellipsoids (96 mm, mus about 19/mm) 5e5  17.9 / 14.3 / 11.1 / 9.96 / 13.0
-inline LaunchShape walk_grid(LaunchShape s, unsigned long long n)
+//               2e6  24.9 / 21.3 / 19.7 / 24.1               5e6  40.0 / 37.2 / 37.9 / 52.5
+//   batch of 16, 6e5 photons in all  13.7 / 11.1 / 9.15 / 8.66    1.2e6  15.4 / 12.9 / 10.8 / 12.4
+//               2.5e6  18.6 / 15.9 / 15.5 / 21.3                  6.2e6  31.2 / 31.9 / 34.1
+inline LaunchShape walk_grid(LaunchShape s, unsigned long long n, const double limits[4])
 {
     if (s.blocks_per_sm < 1) return s;
     const int wpb = s.block / 32, most = s.blocks_per_sm * wpb;
-    const unsigned long long sms = (unsigned long long)(s.grid / s.blocks_per_sm), lane = 32 * sms;
-    int want = 4;
-    if (n > lane * 4 * 26 / 10) want = 8;
-    if (n > lane * 8 * 35 / 10) want = 16;
-    if (n > lane * 16 * 65 / 10) want = 24;
-    if (n > lane * 24 * 13) want = most;
+    const int sms = s.grid / s.blocks_per_sm, warps[5] = {4, 8, 16, 24, most};
+    int k = 0;
+    while (k < 4 && (double)n > limits[k] * (32.0 * sms * warps[k])) ++k;
+    int want = warps[k];
     if (want > most) want = most;
     const int blocks = (want + wpb - 1) / wpb;
-    s.grid = (int)sms * blocks;
+    s.grid = sms * blocks;
     s.warps = (want + blocks - 1) / blocks;
     return s;
 }

@@ -41,9 +41,9 @@ def test_sharing_does_not_change_photons(g, reference, n, block, grid):
     assert balance(r["tally"]) == pytest.approx(n, rel=1e-6)
 
 
-# photon counts at which the grid changes (2.6, 3.5, 6.5 and 13 photons per lane of 4, 8, 16
+# photon counts at which the grid changes (2.6, 3.5, 13 and 26 photons per lane of 4, 8, 16
 # and 24 warps on each of 152 SMs), each against the full grid
-@pytest.mark.parametrize("n", [50585, 50586, 136192, 136193, 505856, 505857, 1517568, 1517569])
+@pytest.mark.parametrize("n", [50585, 50586, 136192, 136193, 1011712, 1011713, 3035136, 3035137])
 @pytest.mark.parametrize("block", [0, 128])
 def test_grid_by_photon_count(g, n, block):
     wl = f32(workloads.c1(n_photons=n).with_(labels=np.ones((8, 8, 8), dtype=np.uint8), src_pos=(4.0, 4.0, 0.0)))
