@@ -490,7 +490,8 @@ mcx_status mcx_run(mcx_sim *s, const mcx_run_cfg *cfg)
     if (cfg->grid_size > 0) shape.grid = cfg->grid_size;
     else if (!claim_static)
         shape = walk_grid(shape, cfg->n_photons,
-                          grid_limits((double)s->nx * s->ny * s->nz * cfg->n_gates * sizeof(double), false));
+                          grid_limits((double)s->nx * s->ny * s->nz * cfg->n_gates * sizeof(double), false),
+                          (double)cfg->dt_ns * cfg->n_gates);
 
     // maps with the walk's one-voxel border, as the label volume
     const uint64_t nvox = (uint64_t)(s->nx + 2) * (s->ny + 2) * (s->nz + 2);

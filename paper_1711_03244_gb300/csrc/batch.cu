@@ -453,7 +453,7 @@ mcx_status mcx_batch_run(mcx_batch *b, const mcx_batch_cfg *cfg)
             photons += sim->n_photons;
             largest = std::max(largest, (double)sim->nx * sim->ny * sim->nz * cfg->n_gates * sizeof(double));
         }
-        shape = walk_grid(shape, photons, grid_limits(largest, true));
+        shape = walk_grid(shape, photons, grid_limits(largest, true), (double)cfg->dt_ns * cfg->n_gates);
     }
     BCUDA(b, cudaEventRecord(b->ev0, stream), "recording an event");
     if (cfg->use_graph) {

@@ -2,6 +2,7 @@
 // (walk.cu).  Not part of the public ABI.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <string>
 #include <cuda_runtime.h>
@@ -122,7 +123,10 @@ struct LaunchShape {
 // stay full for longer and iterate faster.  Too few leave the issue slots idle, and sooner
 // where label loads and deposits go past L2.  So 4, 8, 16 and 24 warps per SM up to so many
 // photons per lane, then all 32: with a map that stays in L2, with a larger one, and for a
-// batch of such maps, whose histories differ most.
+// batch of such maps, whose histories differ most.  The limits hold for windows of 3 ns
+// (650 mm of path in tissue) and more, whose longest histories are 8 to 40 times the mean; a
+// shorter window cuts those and not the mean, so the limits shrink with it (layers, 9.1e5
+// photons, 0.8 ns: 6.3 ms with all warps, 6.8 ms with half).
 constexpr double kGridSmallMap[4] = {2.6, 3.5, 13, 26}, kGridLargeMap[4] = {2.6, 3.5, 6.5, 13},
                  kGridBatch[4] = {2.6, 10, 20, 34};
 constexpr double kGridMapBytes = 128e6;
@@ -142,13 +146,14 @@ inline const double *grid_limits(double map_bytes, bool batch)
 //               2e6  24.9 / 21.3 / 19.7 / 24.1               5e6  40.0 / 37.2 / 37.9 / 52.5
 //   batch of 16, 6e5 photons in all  13.7 / 11.1 / 9.15 / 8.66    1.2e6  15.4 / 12.9 / 10.8 / 12.4
 //               2.5e6  18.6 / 15.9 / 15.5 / 21.3                  6.2e6  31.2 / 31.9 / 34.1
-inline LaunchShape walk_grid(LaunchShape s, unsigned long long n, const double limits[4])
+inline LaunchShape walk_grid(LaunchShape s, unsigned long long n, const double limits[4], double window_ns)
 {
     if (s.blocks_per_sm < 1) return s;
     const int wpb = s.block / 32, most = s.blocks_per_sm * wpb;
     const int sms = s.grid / s.blocks_per_sm, warps[5] = {4, 8, 16, 24, most};
     int k = 0;
-    while (k < 4 && (double)n > limits[k] * (32.0 * sms * warps[k])) ++k;
+    const double scale = std::min(1.0, window_ns / 3.0);
+    while (k < 4 && (double)n > scale * limits[k] * (32.0 * sms * warps[k])) ++k;
     int want = warps[k];
     if (want > most) want = most;
     const int blocks = (want + wpb - 1) / wpb;

@@ -214,7 +214,10 @@ extern "C" mcx_status mcx_run_noalloc(const uint8_t *labels_dev, uint32_t nx, ui
     }
     LaunchShape shape = st.shape;
     if (cfg->grid_size > 0) shape.grid = cfg->grid_size;
-    else shape = walk_grid(shape, cfg->n_photons, grid_limits((double)nx * ny * nz * cfg->n_gates * sizeof(double), false));
+    else
+        shape = walk_grid(shape, cfg->n_photons,
+                          grid_limits((double)nx * ny * nz * cfg->n_gates * sizeof(double), false),
+                          (double)cfg->dt_ns * cfg->n_gates);
     if (shape.grid > kNaMaxBlocks) shape.grid = kNaMaxBlocks;
     unsigned char *scratch = st.scratch;
 
