@@ -31,7 +31,7 @@
 //    lanes at once.  Gate changes, the time limit, the event cap, the roulette and near-axial
 //    directions share one test per segment and a rarely taken path of their own, and one
 //    vote per round covers photons that ended and lanes without one: a scattering iteration
-//    takes about 140 warp instructions instead of 195.  Measured, against testing each
+//    takes an estimated 140 warp instructions (195 counted before).  Measured, against testing each
 //    condition in its own branch and crossing every face at once: two spheres, 2e7 photons
 //    175.6 -> 147 ms; layered tissue, 1e7 photons 87.0 -> 83.2 ms; 24 uneven batched
 //    simulations 57.6 -> 48.8 ms; cube, 3e5 photons 12.8 -> 9.5 ms.
