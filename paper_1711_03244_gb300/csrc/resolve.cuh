@@ -18,29 +18,44 @@ __device__ __forceinline__ T resolved(S v, const float *inv_norm, unsigned label
     return (T)d;
 }
 
+// (float)(v (double)inv) in integers, from the bits of v and inv and with the two roundings of
+// the FP64 way: the 53 x 24-bit product to 53 bits, then to 24, each to nearest even.  False
+// (nothing written) unless v and inv are normal, inv is positive and the result is normal.
+__host__ __device__ __forceinline__ bool fp64_product_to_fp32(unsigned long long v, unsigned inv, unsigned *out)
+{
+    const unsigned ev = (unsigned)(v >> 52) & 0x7ffu, ei = inv >> 23;      // biased by 1023 and 127
+    const unsigned m = inv << 8 | 0x80000000u;                             // inv's 24 bits, in 32
+    const unsigned long long lo = (unsigned long long)(unsigned)v * m;
+    unsigned long long s = ((v >> 32 & 0xfffffu) | 0x100000u) * (unsigned long long)m + (lo >> 32);
+    unsigned rest = (unsigned)lo;                                          // product = s 2^32 + rest
+    int e = (int)(ev + ei) - 1023;                                         // the result's, biased by 127
+    if (s >> 52) {
+        ++e;
+    } else {
+        s = s << 1 | rest >> 31;
+        rest <<= 1;
+    }
+    s += ((unsigned long long)rest + 0x7fffffffu + (unsigned)(s & 1u)) >> 32;
+    // a carry out of either rounding moves into the exponent
+    const unsigned q = (unsigned)((s + 0xfffffffu + (unsigned)(s >> 29 & 1u)) >> 29);
+    if (ev - 1u >= 2046u || ei - 1u >= 254u || (unsigned)(e - 1) >= 253u) return false;
+    *out = ((unsigned)(v >> 32) & 0x80000000u) | (((unsigned)(e - 1) << 23) + q);
+    return true;
+}
+
 // FP64 -> FP32 without the FP64 pipe, whose conversions and product bounded the read-out (2
-// per clock and SM).  v = hi + lo with hi its leading 24 bits and lo the other 29 as 23 and a
-// sticky bit, which rounds as they do: hi + lo is v correctly rounded.  The product with
-// inv_norm keeps its rounding error (FMA) and lo's share, an error below 2^-46 before the one
-// rounding.  Values outside FP32's middle range (and zeros) take the FP64 way.
+// per clock and SM), and with its results: bit for bit, also where FP32 arithmetic would flush
+// the parts of a split product.  Zeros keep FP32's 0 x inv (NaN for an infinite inv); what else
+// the integer way leaves out (results outside FP32's normal range, infinities, NaN) takes the
+// FP64 one.
 template <>
 __device__ __forceinline__ float resolved<float, double, double>(double v, const float *inv_norm, unsigned label)
 {
-    const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
-    const unsigned ex = (h >> 20) & 0x7ffu;                       // biased by 1023
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const float inv = inv_norm ? __ldg(inv_norm + label) : 1.f;
-    // |v| in [2^-60, 2^60), inv in [2^-60, 2^60)
-    const unsigned ei = (__float_as_uint(inv) >> 23) & 0xffu;
-    if (ex - (1023u - 60u) < 120u && ei - (127u - 60u) < 120u) {
-        const unsigned sign = h & 0x80000000u, e8 = (ex - 896u) << 23;
-        const float hi = __uint_as_float(sign | e8 | ((h & 0xfffffu) << 3) | (l >> 29));
-        const unsigned r = (l & 0x1fffffffu) >> 5 | ((l & 0x1fu) ? 1u : 0u);
-        const float lo = __uint2float_rn(r) * __uint_as_float(sign | (e8 - (47u << 23)));   // r 2^(ex - 1023 - 47)
-        if (!inv_norm) return __fadd_rn(hi, lo);
-        const float p = __fmul_rn(hi, inv);
-        return __fadd_rn(p, __fmaf_rn(lo, inv, __fmaf_rn(hi, inv, -p)));
-    }
-    if (v == 0.0) return 0.f;
+    unsigned f;
+    if (fp64_product_to_fp32(b, __float_as_uint(inv), &f)) return __uint_as_float(f);
+    if (!(b << 1)) return __uint_as_float((unsigned)(b >> 32)) * inv;
     return (float)(v * (double)inv);
 }
 

@@ -1,0 +1,73 @@
+"""Rules that the library's host and device code share or that decide a launch, compiled for
+the host and run on the CPU.  No GPU needed."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def compile_and_run(tmp_path, body):
+    """Builds a host program from a body that may use the internal headers; returns its output."""
+    from paper_1711_03244_gb300 import build
+    src, exe = tmp_path / "rule.cu", tmp_path / "rule"
+    src.write_text('#include "resolve.cuh"\n#include <cmath>\n#include <cstdio>\n#include <cstring>\n'
+                   "#include <random>\nusing namespace mcxg;\n" + body)
+    r = subprocess.run([build._nvcc(), "-O2", "-std=c++17", "-I", build.CSRC, "-I", os.path.join(ROOT, "include"),
+                        str(src), "-o", str(exe)] + build.ARCH, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout
+
+
+# the read-out's integer product against the host's FP64 product and conversion: bits of every
+# kind (0), factors of any size whose product is in FP32's range (1), with trailing zeros, as
+# for ties (2), with a power of two and a value on or beside a midpoint of FP32 (3), and with a
+# product on or beside such a midpoint (4)
+@pytest.mark.parametrize("kind", range(5))
+def test_readout_product_equals_fp64(tmp_path, kind):
+    out = compile_and_run(tmp_path, "const int kind = %d;" % kind + r"""
+int main()
+{
+    std::mt19937_64 r(1 + kind);
+    size_t handled = 0, differ = 0, missed = 0;
+    for (int k = 0; k < 10000000; ++k) {
+        unsigned long long v = r();
+        unsigned i = (unsigned)r();
+        if (kind > 0) {
+            const int ei = 1 + (int)(r() % 254), ev = (int)(r() % 256) - 2 - ei + 1023;
+            v = (v & ~(0x7ffull << 52)) | ((unsigned long long)ev << 52);
+            i = (i & 0x7fffffu) | (unsigned)ei << 23;
+        }
+        if (kind == 2) { v &= ~0ull << r() % 52; i &= ~0u << r() % 23; }
+        if (kind == 3) { i &= ~0x7fffffu; v = ((v & ~0x1fffffffull) | 0x10000000ull) + r() % 3 - 1; }
+        float f, want;
+        double d;
+        std::memcpy(&f, &i, 4);
+        if (kind == 4) {
+            const unsigned long long mid = 0x3ffull << 52 | (r() & 0x7fffffull) << 29 | 0x10000000ull;
+            std::memcpy(&d, &mid, 8);
+            d /= f;
+            std::memcpy(&v, &d, 8);
+            v += r() % 5 - 2;
+        }
+        std::memcpy(&d, &v, 8);
+        want = (float)(d * (double)f);
+        unsigned w, got;
+        std::memcpy(&w, &want, 4);
+        if (fp64_product_to_fp32(v, i, &got)) {
+            ++handled;
+            differ += got != w;
+        } else {                            // left to the FP64 way: only at the ends of the range
+            missed += f > 0 && std::isnormal(d) && std::isnormal(f) && std::isnormal(want) &&
+                      std::fabs(want) > 0x1p-125f && std::fabs(want) < 0x1p125f;
+        }
+    }
+    std::printf("%zu %zu %zu\n", handled, differ, missed);
+    return 0;
+}
+""")
+    handled, differ, missed = map(int, out.split())
+    assert handled > (10000 if kind == 0 else 1000000) and differ == 0 and missed == 0

@@ -60,3 +60,65 @@ def test_readout_matches_unpadded_map(g, nx, gates):
         fb = b.fluence(0)
         assert fb.sum(dtype=np.float64) == pytest.approx(ref.sum(), rel=1e-2)
         assert fb.shape == ref.shape and np.isfinite(fb).all()
+
+
+# an absorbing column (1 mean absorption length per voxel, no roulette): its map falls from
+# about 2^13 to 2^-115, and the voxel size and the gate width take the normalisation's factor
+# from 2^63 to 2^-81, so that products reach both far beyond 1 and below FP32's normal range,
+# from factors of all sizes.  The FP32 read-out is the FP64 one rounded once more, bit for bit
+# where the result is a normal number; below, the conversion may flush it.
+@pytest.mark.parametrize("nx", [7, 33])
+@pytest.mark.parametrize("h,dt", [(1e-12, 5.0), (1.0, 5.0), (1.0, 1e8), (1.0, 1e12), (1.0, 1e15), (1e5, 1e10)])
+def test_readout_scales(g, nx, h, dt):
+    import torch
+    ny, nz, n = 5, 80, 20000
+    labels = np.ones((nz, ny, nx), dtype=np.uint8)
+    labels[:, :, ::2] = 2
+    media = np.array([workloads.AIR, (1.0 / h, 0.05 / h, 0.8, 1.37), (1.01 / h, 0.04 / h, 0.8, 1.37)])
+    wl = f32(workloads.c1(n_photons=n).with_(labels=labels, media=media, voxel_mm=h, src_kind=1, waist_mm=2 * h,
+                                             src_pos=(nx * h / 2, 2.5 * h, 0.0), dt_ns=dt))
+    tiny = 2.0 ** -126
+
+    def check(got, m64):
+        want = m64.astype(np.float32)
+        normal = np.abs(want) >= tiny
+        assert np.array_equal(got[normal], want[normal])
+        assert (np.abs(got[~normal]) <= tiny).all()
+        return normal & (want > 0)
+
+    with g.Simulation.from_workload(wl) as sim:
+        sim.run(n, dt_ns=wl.dt_ns, seed=4, rr_threshold=0.0, reflect=0)
+        plain, norm = sim.fluence64(), sim.fluence64(normalized=True)
+        assert check(sim.fluence(), plain).sum() > 400
+        dev = torch.empty((1, nz, ny, nx), device="cuda")
+        sim.fluence(normalized=True, out=dev)
+        compared = check(dev.cpu().numpy(), norm)
+        print(f"products from 2^{np.log2(norm[compared].min()):.0f} to 2^{np.log2(norm[compared].max()):.0f}")
+        assert compared.sum() > 100
+
+
+# the batch's read-out, element by element: against the single run's map (the same photons,
+# as in the batch tests), and its normalisation against its own plain map, from which it
+# differs by the two maps' roundings (FP32 sums are normalised in FP64 and rounded once)
+@pytest.mark.parametrize("accum", [2, 0])
+@pytest.mark.parametrize("nx", [5, 23, 24, 33, 129])
+def test_batch_readout(g, nx, accum):
+    ny, nz, gates, n = 5, 7, 3, 20000
+    labels = np.ones((nz, ny, nx), dtype=np.uint8)
+    labels[nz // 2:, ::2] = 2
+    media = np.array([workloads.AIR, (0.02, 8.0, 0.9, 1.37), (0.1, 3.0, 0.5, 1.37)])
+    wl = f32(workloads.c1(n_photons=n).with_(labels=labels, media=media, src_pos=(nx / 2, 2.5, 0.0)))
+    with g.Simulation.from_workload(wl) as sim:
+        sim.run(n, n_gates=gates, dt_ns=0.05, seed=4)
+        ref = sim.fluence64()
+    with g.Batch() as b:
+        b.add_workload(wl, n_photons=10, seed=3)             # the second map starts elsewhere
+        k = b.add_workload(wl, n_photons=n, seed=4)
+        b.run(n_gates=gates, dt_ns=0.05, accum_mode=accum)
+        plain, norm = b.fluence(k).astype(np.float64), b.fluence(k, normalized=True)
+    assert np.linalg.norm(plain - ref) < 1e-3 * np.linalg.norm(ref)
+    inv = np.zeros(3, dtype=np.float32)
+    for m in (1, 2):
+        inv[m] = 1.0 / (float(np.float32(media[m, 0])) * n * float(np.float32(0.05)))
+    want = plain * inv.astype(np.float64)[labels]
+    assert np.allclose(norm, want, rtol=2.0 ** (-22 if accum == 2 else -23), atol=0)
