@@ -162,6 +162,24 @@ inline LaunchShape walk_grid(LaunchShape s, unsigned long long n, const double l
     return s;
 }
 
+// How a run's photons are shared out: the shape's warps, 32 lanes each, and the caller's
+// claim size; where there are fewer photons than those lanes, each of the shape's warps
+// takes its share in fewer lanes, or (a grid of the caller's) as few warps of each block as
+// hold the block's share.
+inline WalkParams shared_out(WalkParams p, const LaunchShape &s)
+{
+    const unsigned wpb = (unsigned)s.block / 32u, grid = (unsigned)s.grid;
+    p.lanes = 32;
+    p.warps = s.warps > 0 ? (unsigned)s.warps : wpb;
+    if (p.claim_static || p.n_photons >= 32ull * p.warps * grid) return p;
+    // at most 32 warps' worth; counted in 64 bits, since a caller's grid may be of any size
+    const unsigned per_block = p.n_photons ? (unsigned)((p.n_photons + grid - 1ull) / grid) : 1u;
+    if (s.warps <= 0) p.warps = (per_block + 31u) / 32u;
+    p.lanes = (per_block + p.warps - 1u) / p.warps;
+    p.claim_chunk = p.lanes;
+    return p;
+}
+
 // Walk precision: the FP32 product path, or the same kernel in FP64 (trajectory-parity
 // diagnostic; FP64 runs at a small fraction of the FP32 rate on this part).
 enum class Precision { F32 = 0, F64 = 1 };

@@ -1032,23 +1032,6 @@ cudaError_t shape_for(int block, int n_media, int n_det, int tile_e, LaunchShape
     return cudaSuccess;
 }
 
-// How a run's photons are shared out: the shape's warps, 32 lanes each, and the caller's
-// claim size; where there are fewer photons than those lanes, each of the shape's warps
-// takes its share in fewer lanes, or (a grid of the caller's) as few warps of each block as
-// hold the block's share.
-WalkParams shared_out(WalkParams p, const LaunchShape &s)
-{
-    const unsigned wpb = (unsigned)s.block / 32u, grid = (unsigned)s.grid;
-    p.lanes = 32;
-    p.warps = s.warps > 0 ? (unsigned)s.warps : wpb;
-    if (p.claim_static || p.n_photons >= 32ull * p.warps * grid) return p;
-    const unsigned per_block = p.n_photons ? ((unsigned)p.n_photons + grid - 1u) / grid : 1u;
-    if (s.warps <= 0) p.warps = (per_block + 31u) / 32u;
-    p.lanes = (per_block + p.warps - 1u) / p.warps;
-    p.claim_chunk = p.lanes;
-    return p;
-}
-
 template <typename R, bool DET, int ACC, bool ST, bool BATCH = false, bool PAD = true>
 cudaError_t launch(const WalkParams &params, const LaunchShape &s, cudaStream_t st)
 {

@@ -71,3 +71,53 @@ int main()
 """)
     handled, differ, missed = map(int, out.split())
     assert handled > (10000 if kind == 0 else 1000000) and differ == 0 and missed == 0
+
+
+SHARE = r"""
+static WalkParams shared(unsigned long long n, int grid, int block, int warps)
+{
+    LaunchShape s{};
+    s.grid = grid;
+    s.block = block;
+    s.warps = warps;
+    WalkParams p{};
+    p.n_photons = n;
+    p.claim_chunk = 32;
+    return shared_out(p, s);
+}
+"""
+
+
+def test_sharing_of_photons_is_in_range(tmp_path):
+    """Every warp has 1 to 32 lanes and a claim for each, and those lanes hold all photons or
+    are all that there are, whatever the photon count and the caller's grid: also where count
+    and grid add up to more than 32 bits."""
+    out = compile_and_run(tmp_path, SHARE + r"""
+int main()
+{
+    size_t bad = 0, n_cases = 0;
+    std::mt19937_64 r(1);
+    const int grids[] = {1, 2, 152, 608, 4864, 20000, (1 << 24) + 1, 1 << 27, 0x7fffffff};
+    const int blocks[] = {32, 64, 128, 224, 256};
+    for (int grid : grids)
+        for (int block : blocks)
+            for (int warps = 0; warps <= block / 32; ++warps)
+                for (int k = 0; k < 400; ++k) {
+                    const unsigned long long edge[] = {0, 1, 1ull << 32, (1ull << 32) - grid, (1ull << 32) - grid + 1,
+                                                       32ull * grid, 32ull * grid * (block / 32) - 1};
+                    const unsigned long long n = k < 7 ? edge[k] : r() >> (20 + r() % 44);
+                    const WalkParams p = shared(n, grid, block, warps);
+                    const unsigned wpb = block / 32;
+                    const bool range = p.warps >= 1 && p.warps <= wpb && p.lanes >= 1 && p.lanes <= 32 &&
+                                       p.claim_chunk >= p.lanes && (warps == 0 || (int)p.warps == warps);
+                    const bool all = (unsigned long long)p.warps * p.lanes * grid >= n ||
+                                     (p.lanes == 32 && p.warps == (warps ? (unsigned)warps : wpb));
+                    ++n_cases;
+                    bad += !(range && all);
+                }
+    std::printf("%zu %zu\n", n_cases, bad);
+    return 0;
+}
+""")
+    cases, bad = map(int, out.split())
+    assert cases > 50000 and bad == 0
