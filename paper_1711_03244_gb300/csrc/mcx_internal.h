@@ -115,6 +115,7 @@ struct WalkParams {
 struct LaunchShape {
     int grid, block, blocks_per_sm, regs;
     int warps;                        // warps per block that take photons; 0: as the launch finds
+    int resident;                     // blocks that the device holds at once
 };
 
 // The grid of a run of n photons whose caller gives none: as many warps per SM as the run
@@ -165,10 +166,13 @@ inline LaunchShape walk_grid(LaunchShape s, unsigned long long n, const double l
 // How a run's photons are shared out: the shape's warps, 32 lanes each, and the caller's
 // claim size; where there are fewer photons than those lanes, each of the shape's warps
 // takes its share in fewer lanes, or (a grid of the caller's) as few warps of each block as
-// hold the block's share.
+// hold the block's share.  Blocks beyond those that the device holds at once do not count:
+// they start when the others have ended, and find nothing left (a grid of 20 000 blocks, 5e4
+// photons, with its shares counted over all of them: layers 4.7 -> 14.1 ms, cube 7.1 -> 13.7).
 inline WalkParams shared_out(WalkParams p, const LaunchShape &s)
 {
-    const unsigned wpb = (unsigned)s.block / 32u, grid = (unsigned)s.grid;
+    const unsigned wpb = (unsigned)s.block / 32u;
+    const unsigned grid = (unsigned)(s.resident > 0 ? std::min(s.grid, s.resident) : s.grid);
     p.lanes = 32;
     p.warps = s.warps > 0 ? (unsigned)s.warps : wpb;
     if (p.claim_static || p.n_photons >= 32ull * p.warps * grid) return p;

@@ -1026,7 +1026,7 @@ cudaError_t shape_for(int block, int n_media, int n_det, int tile_e, LaunchShape
     if ((e = cudaFuncGetAttributes(&fa, walk_kernel<R, DET, ACC, ST, BATCH, PAD, false>)) != cudaSuccess) return e;
     shape->block = block;
     shape->blocks_per_sm = per_sm;
-    shape->grid = sms * (per_sm > 0 ? per_sm : 1);
+    shape->grid = shape->resident = sms * (per_sm > 0 ? per_sm : 1);
     shape->regs = fa.numRegs;
     shape->warps = 0;
     return cudaSuccess;

@@ -121,3 +121,33 @@ int main()
 """)
     cases, bad = map(int, out.split())
     assert cases > 50000 and bad == 0
+
+
+def test_sharing_ignores_blocks_that_wait(tmp_path):
+    """A grid of more blocks than the device holds shares photons out as one that just fills
+    it; a smaller one by its own blocks."""
+    out = compile_and_run(tmp_path, r"""
+int main()
+{
+    size_t bad = 0;
+    for (int block : {32, 64, 256})
+        for (unsigned long long n = 0; n < 300000; n += 1 + n / 50)
+            for (int grid : {1, 100, 607, 608, 609, 2000, 20000, 0x7fffffff}) {
+                LaunchShape s{}, t{};
+                s.block = t.block = block;
+                s.resident = t.resident = 608;
+                s.grid = grid;
+                t.grid = grid < 608 ? grid : 608;
+                WalkParams p{};
+                p.n_photons = n;
+                p.claim_chunk = 32;
+                const WalkParams a = shared_out(p, s);
+                t.resident = 0;
+                const WalkParams b = shared_out(p, t);
+                bad += a.warps != b.warps || a.lanes != b.lanes || a.claim_chunk != b.claim_chunk;
+            }
+    std::printf("%zu\n", bad);
+    return 0;
+}
+""")
+    assert int(out) == 0
