@@ -18,15 +18,16 @@ __device__ __forceinline__ T resolved(S v, const float *inv_norm, unsigned label
     return (T)d;
 }
 
-// (float)(v (double)inv) in integers, from the bits of v and inv and with the two roundings of
-// the FP64 way: the 53 x 24-bit product to 53 bits, then to 24, each to nearest even.  False
-// (nothing written) unless v and inv are normal, inv is positive and the result is normal.
-__host__ __device__ __forceinline__ bool fp64_product_to_fp32(unsigned long long v, unsigned inv, unsigned *out)
+// (float)(v (double)inv) in integers, from the words of v and the bits of inv and with the two
+// roundings of the FP64 way: the 53 x 24-bit product to 53 bits, then to 24, each to nearest
+// even.  False unless inv is positive and finite and either v is zero or v, inv and the result
+// are normal.
+__host__ __device__ __forceinline__ bool fp64_product_to_fp32(unsigned vhi, unsigned vlo, unsigned inv, unsigned *out)
 {
-    const unsigned ev = (unsigned)(v >> 52) & 0x7ffu, ei = inv >> 23;      // biased by 1023 and 127
+    const unsigned ev = vhi >> 20 & 0x7ffu, ei = inv >> 23;                // biased by 1023 and 127
     const unsigned m = inv << 8 | 0x80000000u;                             // inv's 24 bits, in 32
-    const unsigned long long lo = (unsigned long long)(unsigned)v * m;
-    unsigned long long s = ((v >> 32 & 0xfffffu) | 0x100000u) * (unsigned long long)m + (lo >> 32);
+    const unsigned long long lo = (unsigned long long)vlo * m;
+    unsigned long long s = (vhi & 0xfffffu | 0x100000u) * (unsigned long long)m + (lo >> 32);
     unsigned rest = (unsigned)lo;                                          // product = s 2^32 + rest
     int e = (int)(ev + ei) - 1023;                                         // the result's, biased by 127
     if (s >> 52) {
@@ -38,24 +39,26 @@ __host__ __device__ __forceinline__ bool fp64_product_to_fp32(unsigned long long
     s += ((unsigned long long)rest + 0x7fffffffu + (unsigned)(s & 1u)) >> 32;
     // a carry out of either rounding moves into the exponent
     const unsigned q = (unsigned)((s + 0xfffffffu + (unsigned)(s >> 29 & 1u)) >> 29);
-    if (ev - 1u >= 2046u || ei - 1u >= 254u || (unsigned)(e - 1) >= 253u) return false;
-    *out = ((unsigned)(v >> 32) & 0x80000000u) | (((unsigned)(e - 1) << 23) + q);
-    return true;
+    // asked of the words: asked of the 64 bits, it bounded the read-out like an FP64 comparison
+    // (256 x 256 x 128, 50 gates: 1.63 ms against 1.09)
+    const bool zero = (vhi << 1 | vlo) == 0u && ei < 255u;
+    *out = (vhi & 0x80000000u) | (zero ? 0u : ((unsigned)(e - 1) << 23) + q);
+    return zero || (ev - 1u < 2046u && ei - 1u < 254u && (unsigned)(e - 1) < 253u);
 }
 
 // FP64 -> FP32 without the FP64 pipe, whose conversions and product bounded the read-out (2
 // per clock and SM), and with its results: bit for bit, also where FP32 arithmetic would flush
-// the parts of a split product.  Zeros keep FP32's 0 x inv (NaN for an infinite inv); what else
-// the integer way leaves out (results outside FP32's normal range, infinities, NaN) takes the
-// FP64 one.
+// the parts of a split product.  What the integer way leaves out (results outside FP32's normal
+// range, infinities, NaN) takes the FP64 one.  Zeros do not: a map's empty voxels lie among the
+// others, and with a way of their own nearly every warp took both (64^3, 50 gates, half of the
+// voxels empty: 84 us against 53).
 template <>
 __device__ __forceinline__ float resolved<float, double, double>(double v, const float *inv_norm, unsigned label)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const float inv = inv_norm ? __ldg(inv_norm + label) : 1.f;
     unsigned f;
-    if (fp64_product_to_fp32(b, __float_as_uint(inv), &f)) return __uint_as_float(f);
-    if (!(b << 1)) return __uint_as_float((unsigned)(b >> 32)) * inv;
+    if (fp64_product_to_fp32((unsigned)__double2hiint(v), (unsigned)__double2loint(v), __float_as_uint(inv), &f))
+        return __uint_as_float(f);
     return (float)(v * (double)inv);
 }
 
@@ -90,36 +93,56 @@ resolve_lines(const S *map, unsigned nx, unsigned ny, unsigned lines, unsigned n
         }
 }
 
-// lines too short for a warp: one element per thread
-template <typename T, typename S, typename P>
+// Lines that leave many lanes of a warp idle: E elements per thread, 256 apart.  The divisions
+// for a voxel's line bound the kernel; a plain FP64 -> FP32 conversion runs beside them (33 x
+// 100 x 100, 20 gates: 29 us, in integers 33).
+template <typename T, typename S, typename P, int E>
 __global__ void __launch_bounds__(256)
 resolve_flat(const S *map, unsigned nx, unsigned ny, unsigned nvox, unsigned n_gates, unsigned pnvox,
              const uint8_t *labels, const float *inv_norm, T *out)
 {
-    const size_t total = (size_t)nvox * n_gates, stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += stride) {
-        const unsigned v = (unsigned)(i % nvox), g = (unsigned)(i / nvox);
-        const size_t pv = (size_t)padded_index(v % nx, (v / nx) % ny, v / (nx * ny), nx, ny);
-        out[i] = resolved<T, S, P>(map[(size_t)g * pnvox + pv], inv_norm, labels[pv]);
+    for (unsigned g = blockIdx.y; g < n_gates; g += gridDim.y) {
+        const S *src = map + (size_t)g * pnvox;
+        T *dst = out + (size_t)g * nvox;
+        for (unsigned long long i0 = blockIdx.x * (256ull * E) + threadIdx.x; i0 < nvox; i0 += gridDim.x * (256ull * E)) {
+            S v[E];
+            unsigned b[E];
+#pragma unroll
+            for (int k = 0; k < E; ++k)
+                if (i0 + 256u * k < nvox) {
+                    const unsigned i = (unsigned)i0 + 256u * k, l = i / nx, z = l / ny;
+                    const unsigned pv = (unsigned)padded_index(i - l * nx, l - z * ny, z, nx, ny);
+                    v[k] = __ldcs(src + pv);
+                    b[k] = inv_norm ? __ldg(labels + pv) : 0u;
+                }
+#pragma unroll
+            for (int k = 0; k < E; ++k)
+                if (i0 + 256u * k < nvox)
+                    __stcs(dst + i0 + 256u * k, inv_norm ? resolved<T, S, P>(v[k], inv_norm, b[k]) : (T)v[k]);
+        }
     }
 }
 
-// A warp per line from 24 voxels on (3/4 of its lanes at work).
 template <typename T, typename S, typename P>
 cudaError_t resolve_map(const S *map, unsigned nx, unsigned ny, unsigned nz, unsigned n_gates,
                         const uint8_t *labels, const float *inv_norm, T *out, cudaStream_t st)
 {
     const unsigned lines = ny * nz, nvox = lines * nx;
     const unsigned pnvox = (nx + 2) * (ny + 2) * (nz + 2);
-    if (nx >= 24) {
-        const unsigned gy = std::min(n_gates, 64u);
-        const unsigned gx = std::max(1u, std::min((unsigned)(((unsigned long long)lines + 7) / 8), 152u * 32u / gy));
-        resolve_lines<T, S, P><<<dim3(gx, gy), 256, 0, st>>>(map, nx, ny, lines, n_gates, pnvox, labels, inv_norm, out);
-    } else {
-        const size_t blocks = ((size_t)nvox * n_gates + 255) / 256;
-        resolve_flat<T, S, P><<<(unsigned)std::max<size_t>(1, std::min<size_t>(blocks, 152u * 16u)), 256, 0, st>>>(
-            map, nx, ny, nvox, n_gates, pnvox, labels, inv_norm, out);
-    }
+    const unsigned gy = std::min(n_gates, 64u);
+    auto blocks = [&](unsigned long long n) { return dim3((unsigned)std::max(1ull, std::min(n, 152ull * 32u / gy)), gy); };
+    // A warp per line where more than 3/4 of its lanes have a voxel.  FP64 -> FP32, normalised,
+    // lines / flat: nx = 24 10.6 / 8.5 us, 33 49 / 33, 48 14.7 / 12.6, 64 (50 gates) 53 / 60,
+    // 66 (256 x 256, 50 gates) 1.24 / 0.89 ms, 200 57 / 73 us, 256 (128, 50 gates) 1.11 / 1.71 ms
+    if (4ull * nx > 3ull * ((nx + 31ull) / 32u * 32u))
+        resolve_lines<T, S, P><<<blocks((lines + 7ull) / 8u), 256, 0, st>>>(map, nx, ny, lines, n_gates, pnvox, labels,
+                                                                            inv_norm, out);
+    else if ((unsigned long long)nvox * n_gates > 152ull * 2u * 1024u)
+        resolve_flat<T, S, P, 4><<<blocks((nvox + 1023ull) / 1024u), 256, 0, st>>>(map, nx, ny, nvox, n_gates, pnvox,
+                                                                                   labels, inv_norm, out);
+    else      // too few for two such blocks per SM (16 x 60 x 60, 4 gates: 5.0 us against 6.2)
+        resolve_flat<T, S, P, 1><<<blocks((nvox + 255ull) / 256u), 256, 0, st>>>(map, nx, ny, nvox, n_gates, pnvox,
+                                                                                 labels, inv_norm, out);
     return cudaGetLastError();
 }
 

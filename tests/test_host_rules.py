@@ -57,7 +57,7 @@ int main()
         want = (float)(d * (double)f);
         unsigned w, got;
         std::memcpy(&w, &want, 4);
-        if (fp64_product_to_fp32(v, i, &got)) {
+        if (fp64_product_to_fp32((unsigned)(v >> 32), (unsigned)v, i, &got)) {
             ++handled;
             differ += got != w;
         } else {                            // left to the FP64 way: only at the ends of the range

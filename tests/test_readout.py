@@ -122,3 +122,39 @@ def test_batch_readout(g, nx, accum):
         inv[m] = 1.0 / (float(np.float32(media[m, 0])) * n * float(np.float32(0.05)))
     want = plain * inv.astype(np.float64)[labels]
     assert np.allclose(norm, want, rtol=2.0 ** (-22 if accum == 2 else -23), atol=0)
+
+
+# widths on both sides of the rule (3/4 of a warp's lanes), maps on both sides of the short-line
+# kernel's two forms, and line counts around its tiles, against the same photons in an unpadded map
+@pytest.mark.parametrize("nx,ny,nz,gates", [(1, 1, 1, 1), (3, 1, 2, 1), (48, 9, 7, 3), (49, 9, 7, 3), (65, 64, 3, 2),
+                                            (72, 64, 61, 5), (73, 5, 3, 2), (33, 193, 200, 1), (24, 128, 73, 66)])
+def test_readout_kernels(g, nx, ny, nz, gates):
+    import torch
+    labels = np.ones((nz, ny, nx), dtype=np.uint8)
+    labels[:, :, ::2] = 2
+    media = np.array([workloads.AIR, (0.02, 8.0, 0.9, 1.37), (0.1, 3.0, 0.5, 1.37)])
+    wl = f32(workloads.c1(n_photons=20000).with_(labels=labels, media=media, src_kind=1, waist_mm=max(2.0, ny / 4),
+                                                 src_pos=(nx / 2, ny / 2, 0.0)))
+    with g.Simulation.from_workload(wl) as sim:
+        sim.run(20000, n_gates=gates, dt_ns=0.02, seed=4)
+        plain = sim.fluence64()
+        assert plain.sum() > 0
+        inv = np.zeros(3, dtype=np.float32)
+        for k in (1, 2):
+            inv[k] = 1.0 / (float(np.float32(media[k, 0])) * 20000.0 * float(np.float32(0.02)))
+        want = plain * inv.astype(np.float64)[labels]
+        for normalized, m64 in ((False, plain), (True, want)):
+            assert np.array_equal(sim.fluence64(normalized=normalized), m64)
+            dev = torch.empty((gates, nz, ny, nx), device="cuda")
+            sim.fluence(normalized=normalized, out=dev)
+            assert np.array_equal(dev.cpu().numpy(), m64.astype(np.float32))
+        total = sim.tally()["absorbed"]
+    assert plain.sum() == pytest.approx(total, rel=1e-5)
+    # the same photons into an unpadded map, which is read as it is
+    lab = torch.from_numpy(labels).cuda()
+    flu = torch.empty((gates, nz, ny, nx), device="cuda", dtype=torch.float64)
+    tally = torch.empty(g.NOALLOC_NOUT, device="cuda", dtype=torch.float64)
+    cfg = g.mcx_run_cfg_default(n_photons=20000, n_gates=gates, dt_ns=0.02, seed=4)
+    g.mcx_run_noalloc(lab, wl.voxel_mm, wl.media, wl.src_kind, wl.src_pos, wl.src_dir, wl.waist_mm, cfg, flu, tally)
+    torch.cuda.synchronize()
+    assert np.allclose(plain, flu.cpu().numpy(), rtol=20000 * 2.0 ** -53, atol=0)
