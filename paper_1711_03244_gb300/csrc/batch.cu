@@ -440,20 +440,20 @@ mcx_status mcx_batch_run(mcx_batch *b, const mcx_batch_cfg *cfg)
     LaunchShape shape;
     st = prepare(b, cfg, &shape);
     if (st != MCX_OK) return st;
+    // a recorded run's layout is kept, also for a plain run in between
     uint64_t total = 0;
+    for (const SimHost *sim : b->sims) total += sim->n_photons;
     if (!b->graph) {
-        st = layout(b, cfg, 1.0, b->descs, &total);
+        uint64_t laid_out = 0;
+        st = layout(b, cfg, 1.0, b->descs, &laid_out);
         if (st != MCX_OK) return st;
         b->dirty = false;
     }
     if (cfg->grid_size == 0) {
-        uint64_t photons = 0;
         double largest = 0;
-        for (const SimHost *sim : b->sims) {
-            photons += sim->n_photons;
+        for (const SimHost *sim : b->sims)
             largest = std::max(largest, (double)sim->nx * sim->ny * sim->nz * cfg->n_gates * sizeof(double));
-        }
-        shape = walk_grid(shape, photons, grid_limits(largest, true), (double)cfg->dt_ns * cfg->n_gates);
+        shape = walk_grid(shape, total, grid_limits(largest, true), (double)cfg->dt_ns * cfg->n_gates);
     }
     BCUDA(b, cudaEventRecord(b->ev0, stream), "recording an event");
     if (cfg->use_graph) {

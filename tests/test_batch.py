@@ -194,3 +194,27 @@ def test_batch_members_match_the_oracle(g, orc):
             ob = np.array([orc.run(wl, n_photons=n, photon_offset=(k + 1) * n,
                                    rr_threshold=F32_RR).energy / n for k in range(reps)])
             assert_voxelwise(gr, ob, min_vox=300)
+
+
+@pytest.mark.parametrize("accum", [2, 0])
+def test_batch_switches_between_recorded_and_plain_runs(g, accum):
+    """One batch on one stream of the caller's: each run gives every photon and the same
+    maps, whether it records the graph, replays it or, between replays, does without."""
+    import torch
+    sims = _members()[:4]
+    stream = torch.cuda.Stream()
+    with g.Batch() as b:
+        for wl in sims:
+            b.add_workload(wl)
+        first = None
+        for use_graph in (1, 0, 1, 0, 0, 1):
+            b.run(n_gates=5, dt_ns=1.0, rr_threshold=F32_RR, accum_mode=accum, use_graph=use_graph,
+                  cuda_stream=stream)
+            assert b.stats()["photons"] == sum(w.n_photons for w in sims)
+            maps = [b.fluence(i).astype(np.float64) for i in range(len(sims))]
+            tallies = [b.tally(i) for i in range(len(sims))]
+            for i, wl in enumerate(sims):
+                assert abs(balance(tallies[i]) - wl.n_photons) <= 1e-6 * wl.n_photons
+            first = first or maps
+            for a, m in zip(first, maps):      # the order of the atomic additions differs
+                assert np.allclose(m, a, rtol=1e-6 if accum == 2 else 1e-3, atol=0 if accum == 2 else 1e-6)
