@@ -297,9 +297,11 @@ mcx_status mcx_batch_read_fluence(mcx_batch *b, int32_t id, float *dst, uint64_t
 mcx_status mcx_batch_read_tally(mcx_batch *b, int32_t id, double out[MCX_NTALLY]);
 /* Event counters of the whole batch (MCX_STAT_*). */
 mcx_status mcx_batch_read_stats(mcx_batch *b, uint64_t out[MCX_NSTAT]);
-/* Times the batch with every simulation's photon count scaled by `fraction` (0 < f <= 1)
-   for block sizes {128, 256} x claim chunks {32, 64, 128, 256}, and writes the fastest
-   into cfg (block_size, claim_chunk); best_ms receives its time.  Runs on cfg's stream. */
+/* Times the batch with every simulation's photon count scaled by `fraction` (0 < f <= 1), on
+   the grid that cfg's run of the whole batch takes, for block sizes {128, 256} x claim chunks
+   {32, 64, 128, 256}, and writes the fastest into cfg (block_size, claim_chunk); best_ms
+   receives its time.  Where the scaled photons are fewer than the grid's lanes the chunk has
+   no effect, and 32 is written.  Runs on cfg's stream. */
 mcx_status mcx_batch_autotune(mcx_batch *b, mcx_batch_cfg *cfg, double fraction, float *best_ms);
 int32_t mcx_batch_size(const mcx_batch *b);
 const char *mcx_batch_last_error(const mcx_batch *b);

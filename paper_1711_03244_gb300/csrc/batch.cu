@@ -408,6 +408,14 @@ static mcx_status check_cfg(mcx_batch *b, const mcx_batch_cfg *cfg)
     return MCX_OK;
 }
 
+static uint64_t photons_of(const mcx_batch *b)
+{
+    uint64_t n = 0;
+    for (const SimHost *s : b->sims) n += s->n_photons;
+    return n;
+}
+
+// The launch shape of a run of the whole batch under `cfg`, and the buffers that go with it.
 static mcx_status prepare(mcx_batch *b, const mcx_batch_cfg *cfg, LaunchShape *shape)
 {
     const int block = cfg->block_size ? cfg->block_size : 256;
@@ -418,6 +426,12 @@ static mcx_status prepare(mcx_batch *b, const mcx_batch_cfg *cfg, LaunchShape *s
     BCUDA(b, b->block_tally.ensure((size_t)shape->grid * MCX_NTALLY * sizeof(double)), "allocating");
     BCUDA(b, b->block_stats.ensure((size_t)shape->grid * MCX_NSTAT * 8), "allocating");
     BCUDA(b, b->out_stats.ensure(MCX_NSTAT * 8), "allocating");
+    if (cfg->grid_size == 0) {
+        double largest = 0;
+        for (const SimHost *s : b->sims)
+            largest = std::max(largest, (double)s->nx * s->ny * s->nz * cfg->n_gates * sizeof(double));
+        *shape = walk_grid(*shape, photons_of(b), grid_limits(largest, true), (double)cfg->dt_ns * cfg->n_gates);
+    }
     return MCX_OK;
 }
 
@@ -441,19 +455,12 @@ mcx_status mcx_batch_run(mcx_batch *b, const mcx_batch_cfg *cfg)
     st = prepare(b, cfg, &shape);
     if (st != MCX_OK) return st;
     // a recorded run's layout is kept, also for a plain run in between
-    uint64_t total = 0;
-    for (const SimHost *sim : b->sims) total += sim->n_photons;
+    const uint64_t total = photons_of(b);
     if (!b->graph) {
         uint64_t laid_out = 0;
         st = layout(b, cfg, 1.0, b->descs, &laid_out);
         if (st != MCX_OK) return st;
         b->dirty = false;
-    }
-    if (cfg->grid_size == 0) {
-        double largest = 0;
-        for (const SimHost *sim : b->sims)
-            largest = std::max(largest, (double)sim->nx * sim->ny * sim->nz * cfg->n_gates * sizeof(double));
-        shape = walk_grid(shape, total, grid_limits(largest, true), (double)cfg->dt_ns * cfg->n_gates);
     }
     BCUDA(b, cudaEventRecord(b->ev0, stream), "recording an event");
     if (cfg->use_graph) {
@@ -578,13 +585,14 @@ mcx_status mcx_batch_autotune(mcx_batch *b, mcx_batch_cfg *cfg, double fraction,
             mcx_batch_cfg c = *cfg;
             c.block_size = bl;
             c.claim_chunk = ch;
-            c.grid_size = 0;
-            LaunchShape shape;
+            LaunchShape shape;                        // that of the full run
             st = prepare(b, &c, &shape);
             if (st != MCX_OK) return st;
             uint64_t total = 0;
             st = layout(b, &c, fraction, b->descs_tune, &total);
             if (st != MCX_OK) return st;
+            // with fewer photons than lanes a launch sets its own claims: one trial for all
+            if (ch != chunks[0] && shares_photons(total, shape)) break;
             for (int rep = 0; rep < 2; ++rep) {       // the first pass warms the shape
                 BCUDA(b, cudaEventRecord(b->ev0, stream), "recording an event");
                 st = enqueue(b, &c, b->descs_tune.as<BatchSim>(), total, shape, stream);

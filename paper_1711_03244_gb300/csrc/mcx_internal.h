@@ -169,13 +169,24 @@ inline LaunchShape walk_grid(LaunchShape s, unsigned long long n, const double l
 // hold the block's share.  Blocks beyond those that the device holds at once do not count:
 // they start when the others have ended, and find nothing left (a grid of 20 000 blocks, 5e4
 // photons, with its shares counted over all of them: layers 4.7 -> 14.1 ms, cube 7.1 -> 13.7).
+inline unsigned sharing_blocks(const LaunchShape &s)
+{
+    return (unsigned)(s.resident > 0 ? std::min(s.grid, s.resident) : s.grid);
+}
+inline unsigned sharing_warps(const LaunchShape &s)
+{
+    return s.warps > 0 ? (unsigned)s.warps : (unsigned)s.block / 32u;
+}
+inline bool shares_photons(unsigned long long n, const LaunchShape &s)
+{
+    return n < 32ull * sharing_warps(s) * sharing_blocks(s);
+}
 inline WalkParams shared_out(WalkParams p, const LaunchShape &s)
 {
-    const unsigned wpb = (unsigned)s.block / 32u;
-    const unsigned grid = (unsigned)(s.resident > 0 ? std::min(s.grid, s.resident) : s.grid);
+    const unsigned grid = sharing_blocks(s);
     p.lanes = 32;
-    p.warps = s.warps > 0 ? (unsigned)s.warps : wpb;
-    if (p.claim_static || p.n_photons >= 32ull * p.warps * grid) return p;
+    p.warps = sharing_warps(s);
+    if (p.claim_static || !shares_photons(p.n_photons, s)) return p;
     // at most 32 warps' worth; counted in 64 bits, since a caller's grid may be of any size
     const unsigned per_block = p.n_photons ? (unsigned)((p.n_photons + grid - 1ull) / grid) : 1u;
     if (s.warps <= 0) p.warps = (per_block + 31u) / 32u;

@@ -218,3 +218,41 @@ def test_batch_switches_between_recorded_and_plain_runs(g, accum):
             first = first or maps
             for a, m in zip(first, maps):      # the order of the atomic additions differs
                 assert np.allclose(m, a, rtol=1e-6 if accum == 2 else 1e-3, atol=0 if accum == 2 else 1e-6)
+
+
+def _uneven(n_sims, photons):
+    sims = [f32(w) for w in workloads.c4(n_sims=n_sims)]
+    return [w.with_(n_photons=int(photons * (1 + i % 5) / 3)) for i, w in enumerate(sims)]
+
+
+def test_batch_autotune_times_the_run_it_is_for(g):
+    """With all photons in the trials, the winner's time is that of the run with its settings:
+    nearer to it than to the same run on the full grid, which 6e5 photons of uneven histories
+    do not fill (the time is then that of the longest histories, with more warps beside them)."""
+    with g.Batch() as b:
+        for wl in _uneven(16, 40_000):
+            b.add_workload(wl)
+        best = b.autotune(fraction=1.0, n_gates=5, dt_ns=1.0)
+
+        def ms(**kw):
+            t = []
+            for _ in range(4):
+                b.run(n_gates=5, dt_ns=1.0, block_size=best["block_size"], claim_chunk=best["claim_chunk"], **kw)
+                t.append(b.last_ms())
+            return min(t[1:])
+        # four resident blocks of 256 threads, or eight of 128, on every SM
+        import torch
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        run, full = ms(), ms(grid_size=sms * 1024 // best["block_size"])
+        print(f"trial {best['ms']:.2f} ms, run {run:.2f}, on the full grid {full:.2f}")
+        assert run < 0.85 * full                  # else the two could not be told apart
+        assert best["ms"] < 0.5 * (run + full)
+
+
+@pytest.mark.parametrize("photons,fraction", [(400, 1.0), (2000, 0.5), (4000, 0.25), (20_000, 0.02), (400, 0.1)])
+def test_batch_autotune_keeps_the_default_claim_where_it_has_no_effect(g, photons, fraction):
+    with g.Batch() as b:
+        for wl in _uneven(8, photons):
+            b.add_workload(wl)
+        best = b.autotune(fraction=fraction, n_gates=1, dt_ns=0.2)
+        assert best["claim_chunk"] == 32 and best["block_size"] in (128, 256) and best["ms"] > 0
