@@ -29,7 +29,12 @@ struct Buf {
         release();
         if (want == 0) return cudaSuccess;
         const cudaError_t e = cudaMalloc(&p, want);
-        if (e != cudaSuccess) { p = nullptr; bytes = 0; return e; }
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();         // reported here, not by the next launch's check
+            p = nullptr;
+            bytes = 0;
+            return e;
+        }
         bytes = want;
         return cudaSuccess;
     }

@@ -1636,7 +1636,9 @@ struct DBuf {
     cudaError_t alloc(size_t b)
     {
         bytes = b;
-        return b ? cudaMalloc(&p, b) : cudaSuccess;
+        const cudaError_t e = b ? cudaMalloc(&p, b) : cudaSuccess;
+        if (e != cudaSuccess) (void)cudaGetLastError();   // reported here, not by the next launch's check
+        return e;
     }
     ~DBuf() { if (p) cudaFree(p); }
     template <typename T> T *as() const { return static_cast<T *>(p); }
