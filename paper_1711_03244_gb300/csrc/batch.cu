@@ -580,6 +580,11 @@ mcx_status mcx_batch_autotune(mcx_batch *b, mcx_batch_cfg *cfg, double fraction,
     if (st != MCX_OK) return st;
     if (!(fraction > 0.0) || fraction > 1.0) return bfail(b, MCX_E_ARG, "fraction in (0, 1]");
     if (b->ran) BCUDA(b, cudaEventSynchronize(b->ev1), "waiting for the previous run");
+    // the next run lays out the full batch and records anew, also when a trial fails: trials
+    // write the maps and may move the buffers that a recorded graph points to
+    b->dirty = true;
+    b->ran = false;
+    drop_graph(b);
     cudaStream_t stream = static_cast<cudaStream_t>(cfg->cuda_stream);
     const int blocks[] = {128, 256};
     const int chunks[] = {32, 64, 128, 256};
@@ -613,9 +618,6 @@ mcx_status mcx_batch_autotune(mcx_batch *b, mcx_batch_cfg *cfg, double fraction,
     cfg->block_size = best_block;
     cfg->claim_chunk = best_chunk;
     if (best_ms) *best_ms = best;
-    b->dirty = true;                                  // the next run lays out the full batch
-    b->ran = false;
-    drop_graph(b);
     return MCX_OK;
 }
 

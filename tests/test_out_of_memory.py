@@ -39,3 +39,23 @@ def test_next_call_after_a_refused_run(g):
         c.run(n_gates=1, dt_ns=5.0)
         assert c.stats()["photons"] == 2000
         assert a.stats() == b.stats() and np.allclose(a.fluence(), b.fluence(), rtol=1e-6)
+
+
+def test_recorded_batch_after_a_refused_autotuning(g):
+    """The autotuner's trials have written the maps and moved buffers that the recorded run
+    points to, also when one of them is refused: the next run records anew, and there is no
+    result to read until it has run."""
+    wls = [f32(w).with_(n_photons=20_000) for w in workloads.c4(n_sims=3)]
+    with g.Batch() as b:
+        for wl in wls:
+            b.add_workload(wl)
+        b.run(n_gates=5, dt_ns=1.0, use_graph=1)
+        first = [b.fluence(i) for i in range(len(wls))]
+        refused(g, lambda: b.autotune(n_gates=GATES, dt_ns=1e-9))
+        with pytest.raises(g.McxError) as e:
+            b.stats()
+        assert e.value.status == g.MCX_E_STATE
+        b.run(n_gates=5, dt_ns=1.0, use_graph=1)
+        assert b.stats()["photons"] == 60_000
+        for i, m in enumerate(first):
+            assert np.allclose(b.fluence(i), m, rtol=1e-6, atol=0)
