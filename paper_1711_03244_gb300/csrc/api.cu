@@ -498,6 +498,10 @@ mcx_status mcx_run(mcx_sim *s, const mcx_run_cfg *cfg)
                           grid_limits((double)s->nx * s->ny * s->nz * cfg->n_gates * sizeof(double), false),
                           (double)cfg->dt_ns * cfg->n_gates);
 
+    // from here on the previous results are gone, also when the run fails: an allocation that
+    // is refused has freed the buffer it was to replace
+    s->ran = false;
+
     // maps with the walk's one-voxel border, as the label volume
     const uint64_t nvox = (uint64_t)(s->nx + 2) * (s->ny + 2) * (s->nz + 2);
     const uint64_t nflu = nvox * cfg->n_gates;

@@ -456,6 +456,9 @@ mcx_status mcx_batch_run(mcx_batch *b, const mcx_batch_cfg *cfg)
     if (b->dirty || !b->ran || key != b->graph_key || cfg->accum_mode != b->cfg.accum_mode ||
         cfg->n_gates != b->cfg.n_gates || cfg->order != b->cfg.order)
         drop_graph(b);
+    // from here on the previous results are gone, also when the run fails: an allocation that
+    // is refused has freed the buffer it was to replace
+    b->ran = false;
     LaunchShape shape;
     st = prepare(b, cfg, &shape);
     if (st != MCX_OK) return st;

@@ -59,3 +59,32 @@ def test_recorded_batch_after_a_refused_autotuning(g):
         assert b.stats()["photons"] == 60_000
         for i, m in enumerate(first):
             assert np.allclose(b.fluence(i), m, rtol=1e-6, atol=0)
+
+
+def test_no_result_after_a_refused_run(g):
+    """A run that is refused memory has given up the map of the one before: reading it is
+    refused in turn, until a run succeeds.  Refused arguments leave the results alone."""
+    wl = f32(workloads.c1(n_photons=2000))
+    with g.Simulation.from_workload(wl) as a, g.Batch() as b:
+        b.add_workload(wl)
+        a.run(2000, seed=3)
+        b.run(n_gates=1, dt_ns=5.0)
+        before = a.fluence(), b.fluence(0)
+        for bad in (lambda: a.run(2000, n_gates=0), lambda: b.run(n_gates=0)):
+            with pytest.raises(g.McxError) as e:
+                bad()
+            assert e.value.status == g.MCX_E_ARG
+        a.n_gates = b.n_gates = 1
+        assert np.array_equal(a.fluence(), before[0]) and np.array_equal(b.fluence(0), before[1])
+        for accum in (2, 0):
+            refused(g, lambda: a.run(2000, n_gates=GATES, dt_ns=1e-9, accum_mode=accum))
+            refused(g, lambda: b.run(n_gates=GATES, dt_ns=1e-9, accum_mode=accum))
+            a.n_gates = b.n_gates = 1
+            for read in (a.fluence, a.fluence64, a.tally, a.stats, lambda: b.fluence(0), lambda: b.tally(0), b.stats):
+                with pytest.raises(g.McxError) as e:
+                    read()
+                assert e.value.status == g.MCX_E_STATE
+            a.run(2000, seed=3)
+            b.run(n_gates=1, dt_ns=5.0)
+            assert np.allclose(a.fluence(), before[0], rtol=1e-6)
+            assert np.allclose(b.fluence(0), before[1], rtol=1e-6)
