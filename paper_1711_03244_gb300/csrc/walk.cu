@@ -1024,6 +1024,12 @@ cudaError_t shape_for(int block, int n_media, int n_det, int tile_e, LaunchShape
         return e;
     cudaFuncAttributes fa;
     if ((e = cudaFuncGetAttributes(&fa, walk_kernel<R, DET, ACC, ST, BATCH, PAD, false>)) != cudaSuccess) return e;
+    if constexpr (sizeof(R) == 4 && ACC == kAccF64 && !ST && !BATCH) {
+        // loaded here, not at the first launch for a beam: the allocation-free run may come to
+        // that launch long after it was set up
+        cudaFuncAttributes hot;
+        if ((e = cudaFuncGetAttributes(&hot, walk_kernel<R, DET, ACC, ST, BATCH, PAD, true>)) != cudaSuccess) return e;
+    }
     shape->block = block;
     shape->blocks_per_sm = per_sm;
     shape->grid = shape->resident = sms * (per_sm > 0 ? per_sm : 1);

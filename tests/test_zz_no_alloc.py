@@ -194,3 +194,40 @@ def test_noalloc_refuses_stream_capture(g):
     graph.replay()
     torch.cuda.synchronize()
     assert float(flu.max()) == 1.0
+
+
+LOADS = r"""
+import sys
+sys.path[:0] = [%r, %r]
+import numpy as np, torch
+import paper_1711_03244_gb300 as g, workloads
+from gpu_common import f32
+wl = f32(workloads.paper_b("B1", n_photons=2000))
+labels = torch.from_numpy(wl.labels).cuda()
+flu = torch.empty((1,) + wl.labels.shape, device="cuda", dtype=torch.float64)
+tally = torch.zeros(g.NOALLOC_NOUT, device="cuda", dtype=torch.float64)
+def run(kind):
+    cfg = g.mcx_run_cfg_default(n_photons=2000, dt_ns=5.0, seed=3, reflect=wl.reflect,
+                                cuda_stream=torch.cuda.current_stream())
+    g.mcx_run_noalloc(labels, wl.voxel_mm, wl.media, kind, wl.src_pos, wl.src_dir, 2.0, cfg, flu, tally)
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+free = [run(1), run(1)] + [run(0) for _ in range(3)]
+print(free)
+assert len(set(free[1:])) == 1, free
+"""
+
+
+def test_noalloc_beam_after_another_source_allocates_nothing():
+    """A process whose first calls have a Gaussian source and whose next ones a pencil beam in
+    tissue that scatters little, which runs another instantiation of the walk: no device
+    memory goes after the first call.  In a process of its own, where nothing else has loaded
+    that instantiation."""
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, "-c", LOADS % (os.path.dirname(here), here)], capture_output=True, text=True,
+                       timeout=300)
+    print(r.stdout, r.stderr[-2000:])
+    assert r.returncode == 0
