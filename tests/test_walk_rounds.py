@@ -107,3 +107,50 @@ def test_beam_voxel_sums(g, variant, name, pos, direction, reflect, gates, block
     assert stats[0] == stats[1]
     assert np.array_equal(maps[0] > 0, maps[1] > 0)
     assert np.allclose(maps[0], maps[1], rtol=20000 * 2.0 ** -53, atol=0)
+
+
+# the same sums in the allocation-free run, whose map has no border, on an odd-sized volume, and
+# in a run with detectors, each against its run with every deposit sent to the map
+@pytest.mark.parametrize("pos,direction", [((20.0, 8.0, 0.0), (0.0, 0.0, 1.0)), ((0.0, 5.5, 3.25), (1.0, 0.0, 0.0)),
+                                           ((41.0, 17.0, 23.0), (-0.6, -0.64, -0.48)), ((40.5, 16.5, 22.5), (0.0, 1.0, 0.0))])
+@pytest.mark.parametrize("gates", [1, 3])
+def test_beam_voxel_sums_unpadded(g, pos, direction, gates):
+    import torch
+    labels = np.ones((23, 17, 41), dtype=np.uint8)
+    labels[5:9, 4:12, 10:30] = 2
+    media = np.array([workloads.AIR, (0.01, 1.0, 0.1, 1.37), (0.02, 5.0, 0.8, 1.2)])
+    lab = torch.from_numpy(labels).cuda()
+    maps, tallies = [], []
+    for m in (media, np.concatenate([media, [[0.01, 100.0, 0.9, 1.37]]])):
+        flu = torch.empty((gates,) + labels.shape, device="cuda", dtype=torch.float64)
+        tally = torch.zeros(g.NOALLOC_NOUT, device="cuda", dtype=torch.float64)
+        cfg = g.mcx_run_cfg_default(n_photons=20000, n_gates=gates, dt_ns=0.1, seed=3)
+        g.mcx_run_noalloc(lab, 1.0, m, 0, pos, direction, 0.0, cfg, flu, tally)
+        torch.cuda.synchronize()
+        maps.append(flu.cpu().numpy())
+        tallies.append(tally.cpu().numpy())
+    assert np.array_equal(maps[0] > 0, maps[1] > 0)
+    assert np.allclose(maps[0], maps[1], rtol=20000 * 2.0 ** -53, atol=0)
+    assert np.allclose(tallies[0], tallies[1], rtol=1e-12)
+    wl = f32(workloads.c1(n_photons=20000).with_(labels=labels, media=media, src_pos=pos, src_dir=direction))
+    with g.Simulation.from_workload(wl) as sim:
+        sim.run(20000, n_gates=gates, dt_ns=0.1, seed=3)
+        assert np.allclose(sim.fluence64(), maps[0], rtol=20000 * 2.0 ** -53, atol=0)
+
+
+def test_beam_voxel_sums_with_detectors(g):
+    wl = f32(workloads.paper_b("B2A", n_photons=20000))
+    det = np.array([[30.0, 30.0, 60.0, 15.0], [20.0, 30.0, 0.0, 4.0]])
+    maps, stats, records = [], [], []
+    for media in (wl.media, np.concatenate([wl.media, [[0.01, 100.0, 0.9, 1.37]]])):
+        with g.Simulation.from_workload(wl.with_(media=media, detectors=det)) as sim:
+            sim.run(20000, n_gates=2, dt_ns=0.2, seed=3, max_detected=20000)
+            maps.append(sim.fluence64())
+            stats.append(sim.stats())
+            records.append(sim.detected())
+    assert stats[0] == stats[1] and stats[0]["detected"] > 100
+    assert np.allclose(maps[0], maps[1], rtol=20000 * 2.0 ** -53, atol=0)
+    (a, n), (b, m) = records
+    assert n == m
+    for k in a:                               # the unused medium adds a column of partial paths
+        assert np.array_equal(a[k], b[k][..., :a[k].shape[1]] if k == "ppath" else b[k]), k
