@@ -493,10 +493,14 @@ mcx_status mcx_run(mcx_sim *s, const mcx_run_cfg *cfg)
         shape = it->second;
     }
     if (cfg->grid_size > 0) shape.grid = cfg->grid_size;
-    else if (!claim_static)
+    else if (!claim_static) {
+        GridVolumes v;
+        v.add(s->nx, s->ny, s->nz, s->h, s->n_media, s->props.data(), cfg->n_photons, cfg->n_gates);
         shape = walk_grid(shape, cfg->n_photons,
-                          grid_limits((double)s->nx * s->ny * s->nz * cfg->n_gates * sizeof(double), false),
-                          (double)cfg->dt_ns * cfg->n_gates);
+                          prec == Precision::F64 ? GridUse::F64
+                          : accum == kAccCompensated ? GridUse::Compensated : GridUse::Run,
+                          v, (double)cfg->dt_ns * cfg->n_gates);
+    }
 
     // from here on the previous results are gone, also when the run fails: an allocation that
     // is refused has freed the buffer it was to replace

@@ -91,25 +91,18 @@ struct SimHost {
 };
 
 // Expected work of the longest photon histories of a simulation, for ordering the queue
-// (a scheduling heuristic, not part of the method).  Per label: photons are lost at the
-// rate mua + pi^2 / (L^2 mus') per unit path (absorption, and escape by diffusion from a
-// cube of the grid's mean side L: the slowest mode's loss rate, mus' = mus (1 - g)), so the
-// longest of N photons travels about ln(N) / rate, or up to the time window; times the
-// events per unit path (scatterings mus and voxel crossings 1 / h), weighted by the label's
-// volume fraction.  Starting these photons first keeps them out of the launch's tail.
+// (a scheduling heuristic, not part of the method): longest_history of each label, within the
+// time window, weighted by the label's volume fraction.  Starting these photons first keeps
+// them out of the launch's tail.
 double photon_cost(const SimHost *s, uint32_t n_gates, float dt_ns)
 {
     const double L = s->h * (s->nx + s->ny + s->nz) / 3.0;
     const double ln_n = std::log(std::max<double>((double)s->n_photons, 2.0));
     double c = 0.0;
-    for (uint32_t l = 1; l < s->n_media && l < s->frac.size(); ++l) {
-        if (s->frac[l] <= 0.0) continue;
-        const double mua = s->props[4 * l], mus = s->props[4 * l + 1], g = s->props[4 * l + 2];
-        const double n = s->props[4 * l + 3], musp = std::max(mus * (1.0 - g), 1e-6);
-        const double rate = mua + 9.8696044 / (L * L * musp);
-        const double path = std::min(ln_n / std::max(rate, 1e-9), 299.792458 / n * n_gates * dt_ns);
-        c += s->frac[l] * path * (mus + 1.0 / s->h);
-    }
+    for (uint32_t l = 1; l < s->n_media && l < s->frac.size(); ++l)
+        if (s->frac[l] > 0.0)
+            c += s->frac[l] * longest_history(&s->props[4 * l], s->h, L, ln_n,
+                                              299.792458 / s->props[4 * l + 3] * n_gates * dt_ns);
     return c;
 }
 
@@ -432,10 +425,10 @@ static mcx_status prepare(mcx_batch *b, const mcx_batch_cfg *cfg, LaunchShape *s
     BCUDA(b, b->block_stats.ensure((size_t)shape->grid * MCX_NSTAT * 8), "allocating");
     BCUDA(b, b->out_stats.ensure(MCX_NSTAT * 8), "allocating");
     if (cfg->grid_size == 0) {
-        double largest = 0;
+        GridVolumes v;
         for (const SimHost *s : b->sims)
-            largest = std::max(largest, (double)s->nx * s->ny * s->nz * cfg->n_gates * sizeof(double));
-        *shape = walk_grid(*shape, photons_of(b), grid_limits(largest, true), (double)cfg->dt_ns * cfg->n_gates);
+            v.add(s->nx, s->ny, s->nz, s->h, s->n_media, s->props.data(), s->n_photons, cfg->n_gates);
+        *shape = walk_grid(*shape, photons_of(b), GridUse::Batch, v, (double)cfg->dt_ns * cfg->n_gates);
     }
     return MCX_OK;
 }

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <cuda_runtime.h>
@@ -118,24 +119,56 @@ struct LaunchShape {
     int resident;                     // blocks that the device holds at once
 };
 
+// Expected events of the longest of N photon histories in a medium (ln_n = ln N), in a volume
+// of mean side L, over a path of at most max_path: photons are lost at the rate mua + pi^2 /
+// (L^2 mus') per unit path (absorption, and escape by diffusion from a cube of side L: the
+// slowest mode's loss rate, mus' = mus (1 - g)), so the longest of N travels about ln N / rate;
+// times the events per unit path (scatterings mus and voxel crossings 1 / h).
+inline double longest_history(const float *prop, double h, double L, double ln_n, double max_path)
+{
+    const double mua = prop[0], mus = prop[1], musp = std::max(mus * (1.0 - prop[2]), 1e-6);
+    const double rate = mua + 9.8696044 / (L * L * musp);
+    return std::min(ln_n / std::max(rate, 1e-9), max_path) * (mus + 1.0 / h);
+}
+
+// What the grid's rule asks of a run's volumes: their longest history (over at most 650 mm),
+// whether any of them scatters (mus h >= 0.5), their largest map.
+struct GridVolumes {
+    double longest = 0, map_bytes = 0;
+    bool scatters = false;
+    void add(unsigned nx, unsigned ny, unsigned nz, double h, unsigned n_media, const float *props,
+             unsigned long long n_photons, unsigned n_gates)
+    {
+        const double L = h * ((double)nx + ny + nz) / 3.0, ln_n = std::log(std::max((double)n_photons, 2.0));
+        for (unsigned m = 1; m < n_media; ++m) {
+            longest = std::max(longest, longest_history(props + 4 * m, h, L, ln_n, 650.0));
+            scatters |= props[4 * m + 1] * h >= 0.5;
+        }
+        map_bytes = std::max(map_bytes, (double)nx * ny * nz * n_gates * sizeof(double));
+    }
+};
+enum class GridUse { Run, Compensated, Batch, F64 };
+
 // The grid of a run of n photons whose caller gives none: as many warps per SM as the run
 // keeps busy.  A run ends with its longest histories, and in that time every resident warp
 // still issues the walk for the few lanes it has left; fewer warps take more photons each,
 // stay full for longer and iterate faster.  Too few leave the issue slots idle, and sooner
-// where label loads and deposits go past L2.  So 4, 8, 16 and 24 warps per SM up to so many
+// where label loads and deposits go past L2.  So 8, 16 and 24 warps per SM up to so many
 // photons per lane, then all 32: with a map that stays in L2, with a larger one, and for a
-// batch of such maps, whose histories differ most.  The limits hold for windows of 3 ns
-// (650 mm of path in tissue) and more, whose longest histories are 8 to 40 times the mean; a
-// shorter window cuts those and not the mean, so the limits shrink with it (layers, 9.1e5
-// photons, 0.8 ns: 6.3 ms with all warps, 6.8 ms with half).
-constexpr double kGridSmallMap[4] = {2.6, 3.5, 13, 26}, kGridLargeMap[4] = {2.6, 3.5, 6.5, 13},
-                 kGridBatch[4] = {2.6, 10, 20, 34};
+// batch of such maps, whose histories differ most.  (Four warps pay in the FP64 walk only, which
+// a few warps keep at its rate.)  The limits hold where the longest history is many times the
+// mean, and shrink
+//   with a window below 3 ns (650 mm of path in tissue), which cuts the longest histories and
+//   not the mean (layers, 9.1e5 photons, 0.8 ns: 6.3 ms with all warps, 6.8 ms with half);
+//   where photons cross voxel after voxel without scattering: they wait for label loads, which
+//   only more warps hide (64 mm cube, mus 0.1/mm, 1e6 photons: 2.47 ms at 16 warps, 1.95 at 32);
+//   in the compensated mode, whose sums wait for shared memory, and in batches with the longest
+//   history's length (cube, mua 2/mm, 1e6 photons, compensated: 0.82 ms at 16 warps, 0.60 at
+//   32; 24 such simulations of 8e5 photons in all: 1.06 and 0.81 ms).
+constexpr double kGridSmallMap[4] = {0, 3.5, 13, 26}, kGridLargeMap[4] = {0, 3.5, 6.5, 13},
+                 kGridBatch[4] = {0, 10, 20, 34}, kGridF64[4] = {2.6, 3.5, 13, 26},
+                 kGridCompensated[4] = {0, 3.5, 6.5, 13};
 constexpr double kGridMapBytes = 128e6;
-
-inline const double *grid_limits(double map_bytes, bool batch)
-{
-    return map_bytes > kGridMapBytes ? kGridLargeMap : batch ? kGridBatch : kGridSmallMap;
-}
 // Measured kernel times, ms, at 32 / 24 / 16 / 8 / 4 warps per SM:
 //   cube        2e4  4.23 /  4.22 /  3.93 /  3.93 /  3.75    1e5   7.41 /  6.82 /  5.40 /  4.62 /  5.41
 //               3e5  9.73 /  7.93 /  6.61 /  7.57 / 10.9     1e6  14.0  / 13.2  / 13.2  / 17.6
@@ -147,13 +180,19 @@ inline const double *grid_limits(double map_bytes, bool batch)
 //               2e6  24.9 / 21.3 / 19.7 / 24.1               5e6  40.0 / 37.2 / 37.9 / 52.5
 //   batch of 16, 6e5 photons in all  13.7 / 11.1 / 9.15 / 8.66    1.2e6  15.4 / 12.9 / 10.8 / 12.4
 //               2.5e6  18.6 / 15.9 / 15.5 / 21.3                  6.2e6  31.2 / 31.9 / 34.1
-inline LaunchShape walk_grid(LaunchShape s, unsigned long long n, const double limits[4], double window_ns)
+inline LaunchShape walk_grid(LaunchShape s, unsigned long long n, GridUse use, const GridVolumes &v, double window_ns)
 {
     if (s.blocks_per_sm < 1) return s;
+    const double *limits = use == GridUse::F64 ? kGridF64 : use == GridUse::Compensated ? kGridCompensated
+                         : v.map_bytes > kGridMapBytes ? kGridLargeMap
+                         : use == GridUse::Batch ? kGridBatch : kGridSmallMap;
+    double scale = std::min(1.0, window_ns / 3.0);
+    if (use == GridUse::Batch) scale *= std::min(1.0, v.longest / 4000.0);
+    else if (!v.scatters) scale *= 0.25;
+    if (use == GridUse::Compensated) scale *= std::min(1.0, v.longest / 2000.0);
     const int wpb = s.block / 32, most = s.blocks_per_sm * wpb;
     const int sms = s.grid / s.blocks_per_sm, warps[5] = {4, 8, 16, 24, most};
     int k = 0;
-    const double scale = std::min(1.0, window_ns / 3.0);
     while (k < 4 && (double)n > scale * limits[k] * (32.0 * sms * warps[k])) ++k;
     int want = warps[k];
     if (want > most) want = most;

@@ -214,10 +214,11 @@ extern "C" mcx_status mcx_run_noalloc(const uint8_t *labels_dev, uint32_t nx, ui
     }
     LaunchShape shape = st.shape;
     if (cfg->grid_size > 0) shape.grid = cfg->grid_size;
-    else
-        shape = walk_grid(shape, cfg->n_photons,
-                          grid_limits((double)nx * ny * nz * cfg->n_gates * sizeof(double), false),
-                          (double)cfg->dt_ns * cfg->n_gates);
+    else {
+        GridVolumes v;
+        v.add(nx, ny, nz, voxel_mm, n_media, props, cfg->n_photons, cfg->n_gates);
+        shape = walk_grid(shape, cfg->n_photons, GridUse::Run, v, (double)cfg->dt_ns * cfg->n_gates);
+    }
     if (shape.grid > kNaMaxBlocks) shape.grid = kNaMaxBlocks;
     unsigned char *scratch = st.scratch;
 

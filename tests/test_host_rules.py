@@ -151,3 +151,46 @@ int main()
 }
 """)
     assert int(out) == 0
+
+
+def test_grid_rule(tmp_path):
+    """The grid of a run whose caller gives none: within what the device holds, of warps that a
+    block has, never smaller for more photons, and all of it from some count on; for every use,
+    block size, map, medium and window."""
+    out = compile_and_run(tmp_path, r"""
+int main()
+{
+    size_t bad = 0, cases = 0, steps = 0;
+    const float media[][4] = {{2.f, 5.f, 0.5f, 1.37f}, {0.01f, 10.f, 0.9f, 1.37f}, {0.01f, 0.1f, 0.9f, 1.37f},
+                              {0.f, 0.f, 0.f, 1.f}, {0.f, 20.f, 0.f, 1.4f}};
+    for (GridUse use : {GridUse::Run, GridUse::Compensated, GridUse::Batch, GridUse::F64})
+        for (int block : {32, 64, 96, 128, 224, 256})
+            for (int per_sm : {1, 2, 1024 / block})
+                for (auto &m : media)
+                    for (unsigned gates : {1u, 100000u})
+                        for (double window : {1e-6, 0.1, 2.9, 5.0, 1e6}) {
+                            int last = 0;
+                            for (unsigned long long n = 0; n < (1ull << 40); n = 2 * n + 1 + n / 3) {
+                                const float props[8] = {0, 0, 1, 1, m[0], m[1], m[2], m[3]};
+                                GridVolumes v;
+                                v.add(64, 60, 50, 1.0, 2, props, n, gates);
+                                LaunchShape s{};
+                                s.block = block;
+                                s.blocks_per_sm = per_sm;
+                                s.grid = s.resident = 152 * per_sm;
+                                const LaunchShape t = walk_grid(s, n, use, v, window);
+                                const int warps = t.warps * t.grid;
+                                bad += t.grid < 152 || t.grid > s.grid || t.grid % 152 || t.warps < 1 ||
+                                       t.warps > block / 32 || t.block != block || warps < last;
+                                steps += warps > last;
+                                last = warps;
+                                ++cases;
+                            }
+                            bad += last != 152 * per_sm * (block / 32);
+                        }
+    std::printf("%zu %zu %zu\n", cases, steps, bad);
+    return 0;
+}
+""")
+    cases, steps, bad = map(int, out.split())
+    assert bad == 0 and cases > 50000 and steps > 5000

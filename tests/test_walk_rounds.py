@@ -154,3 +154,48 @@ def test_beam_voxel_sums_with_detectors(g):
     assert n == m
     for k in a:                               # the unused medium adds a column of partial paths
         assert np.array_equal(a[k], b[k][..., :a[k].shape[1]] if k == "ppath" else b[k]), k
+
+
+# the same on both sides of the other limits: a map past L2 (8^3 voxels in 40 000 gates), a short
+# window, the compensated mode, a medium that hardly scatters, the FP64 walk; the counts lie
+# beside the limits of 8, 16 and 24 warps per SM of 152 (FP64: 4)
+GRIDS = {
+    "large map": (dict(gates=40_000, dt=5 / 40_000), [136192, 136193, 505856, 505857, 1517568, 1517569]),
+    "window": (dict(gates=1, dt=0.3), [13619, 13620, 101171, 101172, 303513, 303514]),
+    "compensated": (dict(accum=1), [20_000, 60_000, 250_000, 600_000, 1_600_000]),
+    "clear": (dict(mus=0.1), [34048, 34049, 252928, 252929, 758784, 758785]),
+    "fp64": (dict(precision=1), [20_000, 50585, 50586]),
+}
+
+
+@pytest.mark.parametrize("case,n", [(c, n) for c in GRIDS for n in GRIDS[c][1]])
+def test_grid_does_not_change_photons(g, case, n):
+    kw = GRIDS[case][0]
+    gates, dt = kw.get("gates", 1), kw.get("dt", 5.0)
+    media = np.array([workloads.AIR, (0.01, kw.get("mus", 10.0), 0.9, 1.37)])
+    wl = f32(workloads.c1(n_photons=n).with_(labels=np.ones((8, 8, 8), dtype=np.uint8), media=media,
+                                             src_pos=(4.0, 4.0, 0.0), n_gates=gates, dt_ns=dt))
+    run = dict(exit_log=n, seed=9, accum_mode=kw.get("accum", 2), precision=kw.get("precision", 0))
+    a = gpu_run(wl, **run)
+    b = gpu_run(wl, grid_size=152 * 4, **run)
+    assert a["stats"] == b["stats"] and a["stats"]["photons"] == n
+    assert np.array_equal(a["exits"], b["exits"])
+    assert np.allclose(a["energy"], b["energy"], rtol=1e-6)
+
+
+@pytest.mark.parametrize("n", [389119, 389120, 389121, 1556480, 1556481, 3969024, 3969025])
+def test_batch_grid_does_not_change_photons(g, n):
+    wls = [f32(workloads.c1(n_photons=k).with_(labels=np.ones((16, 16, 16), dtype=np.uint8), src_pos=(8.0, 8.0, 0.0),
+                                               n_gates=1, dt_ns=5.0, seed=k)) for k in (n // 3, n - n // 3)]
+    res = []
+    with g.Batch() as b:
+        for wl in wls:
+            b.add_workload(wl)
+        for kw in ({}, {"grid_size": 152 * 4}):
+            b.run(n_gates=1, dt_ns=5.0, **kw)
+            res.append((b.stats(), [b.tally(i) for i in range(2)], [b.fluence(i) for i in range(2)]))
+    assert res[0][0] == res[1][0] and res[0][0]["photons"] == n
+    for i in range(2):
+        for k in res[0][1][i]:
+            assert res[0][1][i][k] == pytest.approx(res[1][1][i][k], rel=1e-11, abs=1e-11)
+        assert np.allclose(res[0][2][i], res[1][2][i], rtol=1e-6)
