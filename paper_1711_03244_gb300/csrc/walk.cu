@@ -610,8 +610,8 @@ walk_kernel(const WalkParams p)
             if (STATIC) {
                 // the paper's thread-level split: thread g of T takes g, g + T, g + 2T,
                 // ...; the next id follows from the lane's previous one
-                const unsigned long long g0 = blockIdx.x * blockDim.x + threadIdx.x;
-                id = pid == ~0ull ? g0 : pid - p.photon_offset + gridDim.x * blockDim.x;
+                const unsigned long long g0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+                id = pid == ~0ull ? g0 : pid - p.photon_offset + (unsigned long long)gridDim.x * blockDim.x;
             } else if (pool_left >= n) {
                 id = pool_next + rank;
                 pool_next += n;

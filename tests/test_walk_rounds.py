@@ -199,3 +199,13 @@ def test_batch_grid_does_not_change_photons(g, n):
         for k in res[0][1][i]:
             assert res[0][1][i][k] == pytest.approx(res[1][1][i][k], rel=1e-11, abs=1e-11)
         assert np.allclose(res[0][2][i], res[1][2][i], rtol=1e-6)
+
+
+def test_static_split_of_more_threads_than_32_bits_count(g):
+    """The thread-level split over a grid whose threads just exceed 2^32: a thread takes at most
+    one of the photons, and each photon once."""
+    wl = f32(workloads.c1(n_photons=600).with_(labels=np.ones((8, 8, 8), dtype=np.uint8), src_pos=(4.0, 4.0, 0.0)))
+    a = gpu_run(wl, exit_log=600, seed=5)
+    b = gpu_run(wl, exit_log=600, seed=5, claim_mode=1, grid_size=2 ** 24)
+    assert b["stats"] == a["stats"] and np.array_equal(a["exits"], b["exits"])
+    assert balance(b["tally"]) == pytest.approx(600, rel=1e-6)
