@@ -176,7 +176,8 @@ mcx_status mcx_clear_detectors(mcx_sim *sim);
    load-balancing discussion (Fig. 3a), as a dynamic per-warp claim by default.
    Enqueues one simulation on cfg->cuda_stream and returns without waiting.  Zeroes the
    outputs, runs the persistent photon-walk kernel, then reduces the energy tallies.
-   Output buffers are (re)allocated here when the gate count or capacities change. */
+   Output buffers are (re)allocated here when the gate count or capacities change; a run that
+   fails there or later leaves no result to read (refused arguments leave the last one). */
 mcx_status mcx_run(mcx_sim *sim, const mcx_run_cfg *cfg);
 
 /* The host's wait for the device in the workflow (Fig. 1), bounded.
