@@ -38,7 +38,7 @@
 //  * A short run takes fewer warps per SM (walk_grid), and one with fewer photons than lanes
 //    shares them out evenly: its time is that of the longest history, whose warp should
 //    neither wait for warps beside it nor sit on an SM that took most of the photons
-//    (cube, 2e3 / 2e4 / 1e5 / 3e5 photons: 3.5 / 4.5 / 8.2 / 9.7 -> 2.9 / 3.7 / 4.6 / 6.6 ms;
+//    (cube, 2e3 / 2e4 / 1e5 / 3e5 photons: 3.5 / 4.5 / 8.2 / 9.7 -> 2.8 / 3.8 / 4.6 / 6.5 ms;
 //    spread over all warps, a few lanes each: 5.2 ms at 2e4).
 //  * Fast hardware math (MUFU ex2/lg2/sin/cos/rsqrt/rcp) in the FP32 path, the CUDA
 //    analogue of the paper's "native" math optimisation; the same kernel instantiated in
